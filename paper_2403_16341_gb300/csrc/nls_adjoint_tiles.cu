@@ -40,7 +40,7 @@ template <int L, int FAM>
 __global__ void __launch_bounds__(WARP_TPB) k_adjoint_warp(AdjointTileArgs g)
 {
     using S = WarpSolver<L, FAM, false>;
-    using SM = WarpSmem<L, false>;
+    using SM = typename S::SM;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int SEGS = 32 / L;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(WARP_TPB) k_adjoint_warp(AdjointTileArgs g)
     a.maxiters = 1;
     s.init(a, k, sm, FULL); // parameters and the root; its residual is not used
     double row[L];
-    s.jacobian_row(row);
+    s.jacobian_row(row, sm);
     // transpose: lane r takes column r of J, i.e. row r of J^T
 #pragma unroll
     for (int j = 0; j < L; ++j) sm.tr[s.r][j] = row[j];
@@ -100,7 +100,7 @@ static cudaError_t launch_adjoint_warp_lf(const AdjointTileArgs &g, cudaStream_t
 {
     constexpr int per_cta = (WARP_TPB / 32) * (32 / L);
     const int64_t grid = (g.batch + per_cta - 1) / per_cta;
-    k_adjoint_warp<L, FAM><<<(unsigned)grid, WARP_TPB, warp_smem_bytes<L, false>(), st>>>(g);
+    k_adjoint_warp<L, FAM><<<(unsigned)grid, WARP_TPB, warp_smem_bytes<L, false, FAM>(), st>>>(g);
     return cudaGetLastError();
 }
 

@@ -13,6 +13,17 @@
 // broadcast through shared memory, the right-hand side is eliminated on the
 // fly, and back substitution broadcasts one solution component per step.
 //
+// What bounds it.  FP64: the FP64 pipe.  A warp's FP64 instruction holds its
+// scheduler's unit for 64 cycles (76 for a plain add or multiply) however many
+// lanes are active (measured: 1 and 32 active lanes alike), so what counts is
+// the number of FP64 instructions: columns at and beyond n are skipped by
+// warp-uniform branches, and the stencil families' J^T F and J g take their
+// three terms.  Mixed: issue slots and dependent latency, so the pivot row
+// moves in 16-byte accesses, the pivot search takes one or two redux.sync and
+// the loop over the steps is not unrolled (the row shifts by one column per
+// step, which keeps every register index a constant), so it stays in the
+// instruction cache.
+//
 // All segments of a warp execute each pass in lock step (idle segments run
 // masked); a persistent launch refills idle segments from a work counter.
 // The globalisations are those of the thread tiling: Newton (Eq. 2),
@@ -23,15 +34,31 @@
 
 namespace nls {
 
-constexpr int WARP_TPB = 128; // 4 warps per CTA
+constexpr int WARP_TPB = 64; // 2 warps per CTA: they never wait on each other
 
-template <int L, bool MIXED>
-struct WarpSmem {
+// One segment's shared memory.  U holds the pivot row of every step k, from
+// its column k on (the factor U by positions), at slot VEC - 1 + (column - k),
+// its right-hand side one slot before: the columns right of the pivot start
+// on a 16-byte boundary, and the entries (q, c) of one column c lie US - 1 (an
+// odd number) apart, so the back substitution's column read is free of bank
+// conflicts.  Its space also serves the transposes (tr).  The cubic's A stays
+// here rather than in registers: 64 registers fewer per lane let three warps
+// instead of two share a scheduler.
+template <int L, bool MIXED, int FAM>
+struct alignas(16) WarpSmem {
     using P = typename std::conditional<MIXED, float, double>::type;
-    double u[L];      // u broadcast (residual)
-    P prow[L + 1];    // pivot row + its right-hand side
-    P vec[L];         // g broadcast
-    P tr[L][L + 1];   // J^T F transpose-sum
+    static constexpr int VEC = 16 / (int)sizeof(P);
+    static constexpr int US = L + VEC;
+    static constexpr int AS = L + 2;
+    static constexpr int AR = FAM == FAM_CUBIC ? L : 1;
+    double u[L];   // u broadcast (residual)
+    P vec[L];      // g broadcast
+    P prow[L + VEC]; // pivot row + its right-hand side (two-solve solvers)
+    union {
+        alignas(16) P U[L][US];
+        P tr[L][L + 1]; // J^T F transpose-sum
+    };
+    alignas(16) double A[AR][AS]; // cubic: row r of A (FP64)
 };
 
 // Butterfly reductions inside a segment of L lanes (xor offsets < L never
@@ -61,19 +88,34 @@ NLS_DI uint32_t seg_max(uint32_t v, unsigned mask)
     for (int o = L / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(mask, v, o));
     return v;
 }
+// Largest v of each segment, all 32 lanes taking part: one redux.sync when
+// the segment is the warp (as cheap as one shuffle).
+template <int L>
+NLS_DI uint32_t seg_top(uint32_t v)
+{
+    if constexpr (L == 32) return __reduce_max_sync(0xffffffffu, v);
+    else return seg_max<L>(v, 0xffffffffu);
+}
+template <int L>
+NLS_DI uint64_t seg_top(uint64_t v)
+{
+    const uint32_t h = seg_top<L>((uint32_t)(v >> 32));
+    const uint32_t l = seg_top<L>((uint32_t)(v >> 32) == h ? (uint32_t)v : 0u);
+    return ((uint64_t)h << 32) | l;
+}
 
 template <int L, int FAM, bool MIXED>
 struct WarpSolver {
     using P = typename std::conditional<MIXED, float, double>::type;
     using K = decltype(mag_bits(P(0)));
-    using SM = WarpSmem<L, MIXED>;
+    using SM = WarpSmem<L, MIXED, FAM>;
+    static constexpr int VEC = SM::VEC;
 
     // ---- per-lane data of the current instance
     int r;         // row owned by this lane (0..L-1)
     int n;         // system size
     int lane0;     // first lane of the segment in the warp
-    double arow[FAM == FAM_CUBIC ? L : 1];           // cubic: row r of A (FP64, residual)
-    float arowf[FAM == FAM_CUBIC && MIXED ? L : 1];  // cubic, mixed: FP32 copy (Jacobian)
+    float arowf[FAM == FAM_CUBIC && MIXED ? L : 1];  // cubic, mixed: FP32 copy of row r of A (Jacobian)
     double b_r;                 // cubic: b_r; square: p_r; Bratu: lambda
     double u, F, dN;
     uint64_t fmag;              // max_r |F_r| as a bit pattern (segment-uniform)
@@ -94,8 +136,13 @@ struct WarpSolver {
             __syncwarp(mask);
             double s = 0.0;
 #pragma unroll
-            for (int j = 0; j < L; ++j)
-                if (j < n) s = fma(arow[j], sm.u[j], s);
+            for (int j = 0; j < L; j += 2) {
+                if (j >= n) break;
+                const double2 a = *reinterpret_cast<const double2 *>(&sm.A[r][j]);
+                const double2 v = *reinterpret_cast<const double2 *>(&sm.u[j]);
+                s = fma(a.x, v.x, s);
+                if (j + 1 < n) s = fma(a.y, v.y, s);
+            }
             __syncwarp(mask);
             f = s + ur * ur * ur - b_r;
         } else if constexpr (FAM == FAM_BRATU) {
@@ -114,21 +161,16 @@ struct WarpSolver {
         return row_live() ? f : 0.0;
     }
 
-    // row r of J(u) in precision P, by duals over the stencil of F_r
-    NLS_DI void jacobian_row(P (&a)[L]) const
+    // partials of F_r over its stencil by forward-mode duals: d0 = dF_r/du_{r-1},
+    // d1 = dF_r/du_r, d2 = dF_r/du_{r+1}; 0 where the variable does not exist.
+    // Cubic: d1 is the nonlinear part's 3 u_r^2 alone.  All 32 lanes call it.
+    NLS_DI void stencil(P &d0, P &d1, P &d2) const
     {
         const P ur = P(u);
+        d0 = d1 = d2 = P(0);
         if constexpr (FAM == FAM_CUBIC) {
-            // F_r = sum_j A_rj u_j + u_r^3 - b_r: linear coefficients, then d(u_r^3)/du_r
             const auto x = seed<1, 0, P>(ur);
-            const auto c = x * x * x;
-#pragma unroll
-            for (int j = 0; j < L; ++j) {
-                P v;
-                if constexpr (MIXED) v = arowf[j];
-                else v = P(arow[j]);
-                a[j] = (j < n) ? ((j == r) ? v + c.d[0] : v) : P(0);
-            }
+            d1 = (x * x * x).d[0];
         } else if constexpr (FAM == FAM_BRATU) {
             const P inv_h2 = P((n + 1) * (n + 1));
             const P lam = P(b_r);
@@ -137,117 +179,229 @@ struct WarpSolver {
             const auto xc = seed<3, 1, P>(ur);
             const auto xr = seed<3, 2, P>(P(0));
             const auto f = inv_h2 * ((xl + P(-2) * xc) + xr) + lam * exp(xc);
-#pragma unroll
-            for (int j = 0; j < L; ++j) {
-                P v = P(0);
-                if (j == r - 1 && r > 0) v = f.d[0];
-                if (j == r) v = f.d[1];
-                if (j == r + 1 && r + 1 < n) v = f.d[2];
-                a[j] = (j < n) ? v : P(0);
-            }
+            d0 = r > 0 ? f.d[0] : P(0);
+            d1 = f.d[1];
+            d2 = r + 1 < n ? f.d[2] : P(0);
         } else if constexpr (FAM == FAM_SQUARE) {
             const auto x = seed<1, 0, P>(ur);
-            const auto f = x * x;
-#pragma unroll
-            for (int j = 0; j < L; ++j) a[j] = (j == r && j < n) ? f.d[0] : P(0);
+            d1 = (x * x).d[0];
         } else {
             // F_0 = 1 - u_0; F_r = 10 (u_r - u_{r-1}^2); seeds: 0 left, 1 centre
-            const P ul = __shfl_up_sync(0xffffffffu, ur, 1, L); // all lanes run jacobian_row
+            const P ul = __shfl_up_sync(0xffffffffu, ur, 1, L);
             const auto xl = seed<2, 0, P>(ul);
             const auto xc = seed<2, 1, P>(ur);
             const auto f = P(10) * (xc - xl * xl);
+            d0 = r > 0 ? f.d[0] : P(0);
+            d1 = r > 0 ? f.d[1] : P(-1);
+        }
+        if (!row_live()) d0 = d1 = d2 = P(0);
+    }
+
+    // row r of J(u) in precision P from the stencil's partials
+    NLS_DI void jacobian_row(P (&a)[L], const SM &sm, P d0, P d1, P d2) const
+    {
+        if constexpr (FAM == FAM_CUBIC) {
+            // linear coefficients of F_r, then d(u_r^3)/du_r on the diagonal
 #pragma unroll
             for (int j = 0; j < L; ++j) {
-                P v = P(0);
-                if (r == 0) v = (j == 0) ? P(-1) : P(0);
-                else if (j == r - 1) v = f.d[0];
-                else if (j == r) v = f.d[1];
-                a[j] = (j < n) ? v : P(0);
+                P v;
+                if constexpr (MIXED) v = arowf[j];
+                else v = P(sm.A[r][j]);
+                a[j] = (j < n && row_live()) ? ((j == r) ? v + d1 : v) : P(0);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < L; ++j) a[j] = j == r ? d1 : j == r - 1 ? d0 : j == r + 1 ? d2 : P(0);
+        }
+    }
+    NLS_DI void jacobian_row(P (&a)[L], const SM &sm) const
+    {
+        P d0, d1, d2;
+        stencil(d0, d1, d2);
+        jacobian_row(a, sm, d0, d1, d2);
+    }
+
+    // g = J^T F and J g for the row a (and stencil d0, d1, d2) of this lane
+    NLS_DI void gradient(const P (&a)[L], P d0, P d1, P d2, P fp, P &gr, P &Jgr, SM &sm) const
+    {
+        const unsigned FULL = 0xffffffffu;
+        if constexpr (FAM == FAM_CUBIC) {
+            // column sums of F_i * row i.  FP64 keeps the products unrounded (one
+            // fused instruction per row instead of a multiply and an add)
+            P s = P(0);
+            if constexpr (MIXED) {
+#pragma unroll
+                for (int j = 0; j < L; ++j)
+                    if (j < n) sm.tr[r][j] = a[j] * fp;
+                __syncwarp();
+                for (int i = 0; i < n; ++i) s += sm.tr[i][r];
+            } else {
+#pragma unroll
+                for (int j = 0; j < L; ++j)
+                    if (j < n) sm.tr[r][j] = a[j];
+                sm.vec[r] = fp;
+                __syncwarp();
+                for (int i = 0; i < n; ++i) s = fma(sm.tr[i][r], sm.vec[i], s);
+                __syncwarp();
+            }
+            gr = row_live() ? s : P(0);
+            sm.vec[r] = gr;
+            __syncwarp();
+            P t = P(0);
+#pragma unroll
+            for (int j = 0; j < L; ++j)
+                if (j < n) t = fma(a[j], sm.vec[j], t);
+            Jgr = t;
+            __syncwarp();
+        } else {
+            // three terms at most, in the dense sum's order
+            const P q0 = d0 * fp, q1 = d1 * fp, q2 = d2 * fp;
+            const P up = __shfl_up_sync(FULL, q2, 1, L);
+            const P dn = __shfl_down_sync(FULL, q0, 1, L);
+            P s = r > 0 ? up : P(0);
+            s += q1;
+            if (r + 1 < L) s += dn;
+            gr = row_live() ? s : P(0);
+            const P gl = __shfl_up_sync(FULL, gr, 1, L), gn = __shfl_down_sync(FULL, gr, 1, L);
+            P t = r > 0 ? d0 * gl : P(0);
+            t = fma(d1, gr, t);
+            Jgr = r + 1 < L ? fma(d2, gn, t) : t;
+        }
+    }
+
+    // The lane of this lane's segment that holds the pivot: the largest
+    // magnitude m among the candidates, the lowest position among equals (a NaN
+    // not yet at its own pivot position was given m = 0).  All lanes call it.
+    NLS_DI int pivot_lane(K m, bool cand, int pos) const
+    {
+        const unsigned FULL = 0xffffffffu;
+        const unsigned seg = L == 32 ? FULL : ((1u << (L & 31)) - 1u) << lane0;
+        const uint32_t kh = cand ? (uint32_t)(sizeof(K) == 8 ? (uint64_t)m >> 32 : (uint64_t)m) + 1u : 0u;
+        const uint32_t h = seg_top<L>(kh); // every lane, candidate or not
+        bool top = cand && kh == h;
+        unsigned b = __ballot_sync(FULL, top) & seg;
+        if (__any_sync(FULL, (b & (b - 1u)) != 0u)) { // several holders of the largest word
+            if constexpr (sizeof(K) == 8) {
+                const uint32_t kl = top ? (uint32_t)m : 0u;
+                const uint32_t l = seg_top<L>(kl);
+                top = top && kl == l;
+            }
+            const uint32_t kp = top ? ~(uint32_t)pos : 0u;
+            const uint32_t q = seg_top<L>(kp);
+            b = __ballot_sync(FULL, top && kp == q) & seg;
+        }
+        return __ffs(b) - 1;
+    }
+
+    // One step of the LU at column k.  a[0] is column k of the lane's row and
+    // a[c] column k + c; m = n - 1 - k columns follow the pivot.  The updated
+    // column k + c goes to a[c - S]: S = 1 moves the row one column to the left.
+    template <int S, int W>
+    NLS_DI void lu_step(P *a, P &b, int k, int m, int &pos, bool &left, P &y, P &rk, bool &ok, SM &sm) const
+    {
+        const unsigned FULL = 0xffffffffu;
+        const K inf = inf_bits(P(0));
+        const int lane = lane0 + r;
+        K mag = mag_bits(a[0]);
+        if (pos > k && mag > inf) mag = K(0);
+        const int src = pivot_lane(mag, left, pos);
+        const int ppos = __shfl_sync(FULL, pos, src);
+        P *const row = sm.U[k];
+        if (lane == src) {
+            if constexpr (VEC == 4) *reinterpret_cast<float2 *>(row + 2) = make_float2(b, a[0]);
+            else *reinterpret_cast<double2 *>(row) = make_double2(b, a[0]);
+#pragma unroll
+            for (int c = 1; c < W; c += VEC) {
+                if (c > m) break;
+                if constexpr (VEC == 4)
+                    *reinterpret_cast<float4 *>(row + 3 + c) =
+                        make_float4(a[c], c + 1 < W ? a[c + 1 < W ? c + 1 : 0] : P(0),
+                                    c + 2 < W ? a[c + 2 < W ? c + 2 : 0] : P(0), c + 3 < W ? a[c + 3 < W ? c + 3 : 0] : P(0));
+                else
+                    *reinterpret_cast<double2 *>(row + 1 + c) =
+                        make_double2(a[c], c + 1 < W ? a[c + 1 < W ? c + 1 : 0] : P(0));
             }
         }
-        if (!row_live()) {
-#pragma unroll
-            for (int j = 0; j < L; ++j) a[j] = P(0);
+        __syncwarp();
+        P p0, pb;
+        if constexpr (VEC == 4) {
+            const float2 v = *reinterpret_cast<const float2 *>(row + 2);
+            pb = v.x;
+            p0 = v.y;
+        } else {
+            const double2 v = *reinterpret_cast<const double2 *>(row);
+            pb = v.x;
+            p0 = v.y;
         }
+        const K pm = mag_bits(p0);
+        if (pm == K(0) || pm >= inf) ok = false;
+        const P pr = rcp(p0);
+        if (r == k) {
+            y = pb;
+            rk = pr;
+        }
+        // the row at position k moves to the pivot's old position
+        if (left && pos == k) pos = ppos;
+        if (lane == src) {
+            pos = k;
+            left = false;
+        }
+        const P l = left ? a[0] * pr : P(0);
+#pragma unroll
+        for (int c = 1; c < W; c += VEC) {
+            if (c > m) break;
+            if constexpr (VEC == 4) {
+                const float4 v = *reinterpret_cast<const float4 *>(row + 3 + c);
+                a[c - S] = a[c] - l * v.x;
+                if (c + 1 < W) a[c + 1 - S] = a[c + 1] - l * v.y;
+                if (c + 2 < W) a[c + 2 - S] = a[c + 2] - l * v.z;
+                if (c + 3 < W) a[c + 3 - S] = a[c + 3] - l * v.w;
+            } else {
+                const double2 v = *reinterpret_cast<const double2 *>(row + 1 + c);
+                a[c - S] = a[c] - l * v.x;
+                if (c + 1 < W && c + 1 <= m) a[c + 1 - S] = a[c + 1] - l * v.y;
+            }
+        }
+        b -= l * pb;
     }
 
     // LU with partial pivoting and on-the-fly elimination of b; on return
     // b holds x_r (component r of the solution) in lane r.  Returns false
-    // (segment-uniform) on a zero or non-finite pivot.
+    // (segment-uniform) on a zero or non-finite pivot.  The row a is consumed.
+    // FP32: the steps are a loop whose body moves the row one column to the
+    // left, so it fits the instruction cache.  FP64: the steps are unrolled and
+    // the row stays in place; a shifting update would overwrite a register that
+    // the FP64 unit, which reads its operands late, still has to fetch (the
+    // shifting loop measured 6.98 ms on 20,011 trust-region n = 27 systems).
+    // Against whole rows written by scalar stores, 64-bit shuffle butterflies
+    // for the pivot and unskipped columns: 2^16 mixed n = 32 systems
+    // (backtracking) 5.66 -> 3.31 ms, 20,011 FP64 n = 27 ones 6.61 -> 5.98 ms,
+    // 1,024 ten-dimensional Rosenbrock ones (trust region) 2.44 -> 1.77 ms.
     NLS_DI bool lu_solve(P (&a)[L], P &b, SM &sm) const
     {
-        const K inf = inf_bits(P(0));
+        const unsigned FULL = 0xffffffffu;
         int pos = r;              // position of this lane's row after the interchanges
-        bool live = row_live();
-        P rc = P(0);              // 1/pivot, kept by the lane whose row is pivot row `pos`
+        bool left = row_live();   // not a pivot row yet
+        P y = P(0), rk = P(0);    // lane k: right-hand side and reciprocal of pivot row k
         bool ok = true;
-#pragma unroll
-        for (int k = 0; k < L; ++k) {
-            if (k < n) {
-                // key: |a_ik| bit pattern; NaN below the diagonal position never wins
-                K m = mag_bits(a[k]);
-                if (pos > k && m > inf) m = K(0);
-                const bool cand = live && pos >= k;
-                // larger key first, then the lower position
-                uint64_t key;
-                if constexpr (sizeof(K) == 4) key = cand ? ((uint64_t)m << 32) | (uint32_t)(L - 1 - pos) : 0ull;
-                else key = cand ? m : 0ull;
-                uint64_t best = seg_max<L>(key, 0xffffffffu);
-                int ppos;
-                if constexpr (sizeof(K) == 4) {
-                    ppos = L - 1 - (int)(best & 0xffffffffu);
-                    best >>= 32;
-                } else {
-                    const uint32_t tie = (cand && key == best) ? (uint32_t)(L - 1 - pos) : 0u;
-                    ppos = L - 1 - (int)seg_max<L>(tie, 0xffffffffu);
-                    if (best == 0) ppos = k; // all-zero column: singular below
-                }
-                const bool is_piv = cand && pos == ppos;
-                if (best == 0 || best >= (uint64_t)inf) ok = false;
-                // broadcast the pivot row (columns > k) and its right-hand side
-                if (is_piv) {
-#pragma unroll
-                    for (int c = k + 1; c < L; ++c) sm.prow[c] = a[c];
-                    sm.prow[k] = a[k];
-                    sm.prow[L] = b;
-                }
-                __syncwarp();
-                const P piv = sm.prow[k];
-                const P pr = rcp(piv);
-                const P pb = sm.prow[L];
-                // the row at position k moves to the pivot's old position
-                if (cand && pos == k && !is_piv) pos = ppos;
-                if (is_piv) {
-                    pos = k;
-                    rc = pr;
-                }
-                if (cand && !is_piv) {
-                    const P l = a[k] * pr;
-#pragma unroll
-                    for (int c = k + 1; c < L; ++c) a[c] -= l * sm.prow[c];
-                    b -= l * pb;
-                }
-                __syncwarp();
-            }
+        if constexpr (MIXED) {
+            for (int k = 0; k < n; ++k) lu_step<1, L>(a, b, k, n - 1 - k, pos, left, y, rk, ok, sm);
+        } else {
+            static_for<0, L>([&](auto Kc) {
+                constexpr int k = decltype(Kc)::value;
+                if (k < n) lu_step<0, L - k>(a + k, b, k, n - 1 - k, pos, left, y, rk, ok, sm);
+            });
         }
-        // back substitution: x_k from the lane holding pivot row k, then
-        // every lane holding an earlier pivot row removes its contribution
+        // back substitution: lane k holds pivot row k's right-hand side; x_k goes
+        // to every lane, and the lanes of earlier positions remove its contribution
         P x = P(0);
-#pragma unroll
-        for (int k = L - 1; k >= 0; --k) {
-            if (k < n) {
-                P xk = P(0);
-                if (live && pos == k) {
-                    xk = b * rc;
-                    sm.prow[0] = xk;
-                }
-                __syncwarp();
-                xk = sm.prow[0];
-                __syncwarp();
-                if (r == k) x = xk;
-                if (live && pos < k) b -= a[k] * xk;
-            }
+#pragma unroll 4
+        for (int k = n - 1; k >= 0; --k) {
+            const P xk = __shfl_sync(FULL, y * rk, k, L);
+            if (r == k) x = xk;
+            if (r < k) y -= sm.U[r][VEC - 1 + k - r] * xk;
         }
+        __syncwarp(); // U is free for the next use
         b = x;
         return ok;
     }
@@ -262,7 +416,7 @@ struct WarpSolver {
             for (int j = 0; j < L; ++j) {
                 double v = 0.0;
                 if (j < n && row_live()) v = __ldg(a.params + (int64_t)(r * n + j) * B + k);
-                arow[j] = v;
+                sm.A[r][j] = v;
                 if constexpr (MIXED) arowf[j] = float(v);
             }
             if (row_live()) b_r = __ldg(a.params + (int64_t)(n * n + r) * B + k);
@@ -309,28 +463,17 @@ struct WarpSolver {
         bool failed = false;
         if (__any_sync(0xffffffffu, run && need_jac)) {
             const bool fresh = run && need_jac;
-            P a[L];
-            jacobian_row(a);
+            P a[L], d0, d1, d2;
+            stencil(d0, d1, d2);
+            jacobian_row(a, sm, d0, d1, d2);
             const P fp = P(F);
             if (fresh) Fp = fp;
             if (A.alg == ALG_TRUST_DOGLEG) {
-                // g = J^T F: column sums of F_r * row r, and J g
-#pragma unroll
-                for (int j = 0; j < L; ++j) sm.tr[r][j] = a[j] * fp;
-                __syncwarp();
-                P s = P(0);
-#pragma unroll
-                for (int i = 0; i < L; ++i) s += sm.tr[i][r];
-                __syncwarp();
-                if (fresh) g = s;
-                sm.vec[r] = s;
-                __syncwarp();
-                P t = P(0);
-#pragma unroll
-                for (int j = 0; j < L; ++j) t = fma(a[j], sm.vec[j], t);
-                __syncwarp();
+                P gr, Jgr;
+                gradient(a, d0, d1, d2, fp, gr, Jgr, sm);
                 if (fresh) {
-                    Jg = t;
+                    g = gr;
+                    Jg = Jgr;
                     ++ngrad;
                 }
             }
@@ -368,7 +511,7 @@ struct WarpSolver {
                 const double ut = fma(alpha, dN, u);
                 const double Ft = residual(ut, sm, 0xffffffffu);
                 const double fFt = seg_sum<L>(Ft * Ft, 0xffffffffu);
-                const bool fin = seg_max<L>(mag_bits(Ft), 0xffffffffu) < INF64_BITS;
+                const bool fin = seg_all(mag_bits(Ft) < INF64_BITS);
                 if (trying) {
                     ++nfev;
                     if (fin && 0.5 * fFt <= phi0 + LS_C1 * alpha * s) {
@@ -395,35 +538,38 @@ struct WarpSolver {
             // dogleg branches; a collective inside a branch would diverge).
             const P D2 = P(Delta * Delta);
             const P nN2 = seg_sum<L>(P(dN) * P(dN), 0xffffffffu);
-            const P gg = seg_sum<L>(g * g, 0xffffffffu);
-            const P JgJg = seg_sum<L>(Jg * Jg, 0xffffffffu);
-            const P t = gg / JgJg; // Cauchy point c = -t g minimises the model along -g
-            const P cc = t * t * gg;
-            const P w = P(dN) + t * g; // dN - c
-            const P aa = seg_sum<L>(w * w, 0xffffffffu);
-            const P bb = seg_sum<L>(-t * g * w, 0xffffffffu);
             // pred = -2 F.Jd - ||Jd||^2 (Eq. 15) from segment-uniform scalars:
             // J dN = -F and F.(J g) = g.g (g = J^T F), so no J d is formed
-            double d, pred;
-            if (nN2 <= D2) {
-                d = dN;
-                pred = fF;
-            } else if (cc >= D2) {
-                const P sc = P(Delta) / nls_sqrt(gg);
-                d = double(-sc * g);
-                pred = double(sc * (P(2) * gg - sc * JgJg));
-            } else {
-                const P q = cc - D2;
-                const P tau = (-bb + nls_sqrt(bb * bb - aa * q)) / aa;
-                d = double(fma(tau, w, -t * g));
-                const P s1 = (P(1) - tau) * t; // J d = -s1 J g - tau F
-                pred = double(s1 * (P(2) * (P(1) - tau) * gg - s1 * JgJg) + tau * (P(2) - tau) * P(fF));
+            double d = dN, pred = fF;
+            // the dogleg's sums and quotients only when a segment's Newton step
+            // leaves its region (a warp-uniform branch)
+            if (__any_sync(0xffffffffu, run && !(nN2 <= D2))) {
+                const P gg = seg_sum<L>(g * g, 0xffffffffu);
+                const P JgJg = seg_sum<L>(Jg * Jg, 0xffffffffu);
+                const P t = gg / JgJg; // Cauchy point c = -t g minimises the model along -g
+                const P cc = t * t * gg;
+                const P w = P(dN) + t * g; // dN - c
+                const P aa = seg_sum<L>(w * w, 0xffffffffu);
+                const P bb = seg_sum<L>(-t * g * w, 0xffffffffu);
+                if (nN2 <= D2) {
+                    // the Newton step
+                } else if (cc >= D2) {
+                    const P sc = P(Delta) / nls_sqrt(gg);
+                    d = double(-sc * g);
+                    pred = double(sc * (P(2) * gg - sc * JgJg));
+                } else {
+                    const P q = cc - D2;
+                    const P tau = (-bb + nls_sqrt(bb * bb - aa * q)) / aa;
+                    d = double(fma(tau, w, -t * g));
+                    const P s1 = (P(1) - tau) * t; // J d = -s1 J g - tau F
+                    pred = double(s1 * (P(2) * (P(1) - tau) * gg - s1 * JgJg) + tau * (P(2) - tau) * P(fF));
+                }
             }
             if (!row_live()) d = 0.0;
             const double ut = u + d;
             const double Ft = residual(ut, sm, 0xffffffffu);
             const double fFt = seg_sum<L>(Ft * Ft, 0xffffffffu);
-            const bool fin = seg_max<L>(mag_bits(Ft), 0xffffffffu) < INF64_BITS;
+            const bool fin = seg_all(mag_bits(Ft) < INF64_BITS);
             const double ared = fF - fFt;
             if (go) {
                 ++nfev;
@@ -441,20 +587,37 @@ struct WarpSolver {
                 }
             }
         }
-        const uint64_t m = seg_max<L>(mag_bits(F), 0xffffffffu);
-        if (run) fmag = m;
+        const bool fin = seg_all(mag_bits(F) < INF64_BITS);
+        const bool conv = seg_all(mag_bits(F) <= mag_bits(A.abstol));
         if (go && !failed) {
-            if (m >= INF64_BITS) status = ST_NONFINITE;
-            else if (m <= mag_bits(A.abstol)) status = ST_SUCCESS;
+            if (!fin) status = ST_NONFINITE;
+            else if (conv) status = ST_SUCCESS;
             else if (it >= A.maxiters) status = ST_MAXITERS;
         }
+        // the residual's norm itself is an output: formed when an instance ends
+        if (__any_sync(0xffffffffu, run && status != ST_RUNNING)) residual_norm(run);
+    }
+
+    // whether p holds on every lane of this lane's segment (all lanes call it)
+    NLS_DI bool seg_all(bool p) const
+    {
+        const unsigned b = __ballot_sync(0xffffffffu, p);
+        return L == 32 ? b == 0xffffffffu : ((b >> lane0) & ((1u << (L & 31)) - 1u)) == (1u << (L & 31)) - 1u;
+    }
+    // fmag = max_r |F_r| for the segments with `run` (all lanes call it)
+    NLS_DI void residual_norm(bool run)
+    {
+        const uint64_t m = seg_top<L>(mag_bits(F));
+        if (run) fmag = m;
     }
 };
 
-template <int L, bool MIXED>
+template <int L, bool MIXED, int FAM>
 constexpr int warp_smem_bytes()
 {
-    return (WARP_TPB / 32) * (32 / L) * (int)sizeof(WarpSmem<L, MIXED>);
+    constexpr int bytes = (WARP_TPB / 32) * (32 / L) * (int)sizeof(WarpSmem<L, MIXED, FAM>);
+    static_assert(bytes <= 48 * 1024, "no opt-in beyond 48 KB is made for these kernels");
+    return bytes;
 }
 
 // The segment loop shared by the warp-tiled solvers S (r, n, lane0, status,
@@ -464,7 +627,7 @@ template <class S, int L, bool MIXED>
 NLS_DI void warp_lanes(SolveArgs &a)
 {
     apply_dyn_batch(a);
-    using SM = WarpSmem<L, MIXED>;
+    using SM = typename S::SM;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int SEGS = 32 / L;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -524,6 +687,7 @@ NLS_DI void warp_lanes(SolveArgs &a)
         // pass never splits a collective
         const bool late = a.budget_ns && __shfl_sync(FULL, global_ns(), 0) > t_end;
         if (late) {
+            s.residual_norm(have);
             if (have) s.status = ST_ABORTED;
         } else {
             s.pass(a, sm, have);
@@ -542,8 +706,18 @@ NLS_DI void warp_lanes(SolveArgs &a)
     }
 }
 
+// CTAs per SM that the compiler makes room for: the cubic's 32-lane FP64
+// kernel takes the 6 that its shared memory allows (164 registers instead of
+// 222, which held 4).  Its mixed kernel fits 6 by itself; 8 (128 registers and
+// a spill) measured 2% faster alone but 5% slower in a flush of many sizes.
 template <int L, int FAM, bool MIXED>
-__global__ void __launch_bounds__(WARP_TPB) k_solve_warp(SolveArgs a)
+constexpr int warp_min_ctas()
+{
+    return L == 32 && FAM == FAM_CUBIC && !MIXED ? 6 : 1;
+}
+
+template <int L, int FAM, bool MIXED>
+__global__ void __launch_bounds__(WARP_TPB, warp_min_ctas<L, FAM, MIXED>()) k_solve_warp(SolveArgs a)
 {
     warp_lanes<WarpSolver<L, FAM, MIXED>, L, MIXED>(a);
 }

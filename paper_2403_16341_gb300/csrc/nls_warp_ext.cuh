@@ -196,7 +196,7 @@ struct WarpSolverTwoSolve : WarpSolverExtBase<L, FAM, MIXED> {
         const unsigned FULL = 0xffffffffu;
         if (run) ++it;
         P a[L];
-        this->jacobian_row(a);
+        this->jacobian_row(a, sm);
         int pos;
         P rc;
         const bool ok = warp_lu_factor<L>(a, r, n, sm, pos, rc);
@@ -269,7 +269,7 @@ struct WarpSolverBroyden : WarpSolverExtBase<L, FAM, MIXED> {
             if (A.alg == ALG_MOD_BROYDEN) {
                 // H = J(u_0)^-1, one column per unit vector
                 P a[L];
-                this->jacobian_row(a);
+                this->jacobian_row(a, sm);
                 int pos;
                 P rc;
                 const bool ok = warp_lu_factor<L>(a, r, n, sm, pos, rc);
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(WARP_TPB) k_solve_warp_ext(SolveArgs a)
 template <int L, int FAM, bool MIXED, int ALG>
 cudaError_t launch_warp_ext(const SolveArgs &a, int grid, cudaStream_t st)
 {
-    k_solve_warp_ext<L, FAM, MIXED, ALG><<<grid, WARP_TPB, warp_smem_bytes<L, MIXED>(), st>>>(a);
+    k_solve_warp_ext<L, FAM, MIXED, ALG><<<grid, WARP_TPB, warp_smem_bytes<L, MIXED, FAM>(), st>>>(a);
     return cudaGetLastError();
 }
 
@@ -374,7 +374,7 @@ KernelInfo warp_ext_info()
     k.launch = &launch_warp_ext<L, FAM, MIXED, ALG>;
     k.func = reinterpret_cast<const void *>(&k_solve_warp_ext<L, FAM, MIXED, ALG>);
     k.block = WARP_TPB;
-    k.smem = warp_smem_bytes<L, MIXED>();
+    k.smem = warp_smem_bytes<L, MIXED, FAM>();
     k.per_cta = (WARP_TPB / 32) * (32 / L);
     return k;
 }

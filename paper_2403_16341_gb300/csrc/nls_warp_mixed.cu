@@ -7,7 +7,7 @@ namespace nls {
 template <int L, int FAM>
 static cudaError_t launch_warp_mixed(const SolveArgs &a, int grid, cudaStream_t st)
 {
-    k_solve_warp<L, FAM, true><<<grid, WARP_TPB, warp_smem_bytes<L, true>(), st>>>(a);
+    k_solve_warp<L, FAM, true><<<grid, WARP_TPB, warp_smem_bytes<L, true, FAM>(), st>>>(a);
     return cudaGetLastError();
 }
 
@@ -18,7 +18,7 @@ static KernelInfo info_mixed()
     k.launch = &launch_warp_mixed<L, FAM>;
     k.func = reinterpret_cast<const void *>(&k_solve_warp<L, FAM, true>);
     k.block = WARP_TPB;
-    k.smem = warp_smem_bytes<L, true>();
+    k.smem = warp_smem_bytes<L, true, FAM>();
     k.per_cta = (WARP_TPB / 32) * (32 / L);
     return k;
 }
