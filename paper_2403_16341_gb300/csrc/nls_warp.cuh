@@ -706,18 +706,16 @@ NLS_DI void warp_lanes(SolveArgs &a)
     }
 }
 
-// CTAs per SM that the compiler makes room for: the cubic's 32-lane FP64
-// kernel takes the 6 that its shared memory allows (164 registers instead of
-// 222, which held 4).  Its mixed kernel fits 6 by itself; 8 (128 registers and
-// a spill) measured 2% faster alone but 5% slower in a flush of many sizes.
-template <int L, int FAM, bool MIXED>
-constexpr int warp_min_ctas()
-{
-    return L == 32 && FAM == FAM_CUBIC && !MIXED ? 6 : 1;
-}
+// CTAs per SM that the compiler makes room for (0: its own choice).  The
+// 32-lane FP64 kernels take the 6 that the cubic's shared memory allows (164
+// registers instead of 222, which held 4).  Mixed, 8 CTAs (128 registers and a
+// spill) measured 2% faster on n = 32 alone but 5% slower in a flush of many
+// sizes.
+template <int L, bool MIXED>
+constexpr int warp_min_ctas() { return L == 32 && !MIXED ? 6 : 0; }
 
 template <int L, int FAM, bool MIXED>
-__global__ void __launch_bounds__(WARP_TPB, warp_min_ctas<L, FAM, MIXED>()) k_solve_warp(SolveArgs a)
+__global__ void __launch_bounds__(WARP_TPB, warp_min_ctas<L, MIXED>()) k_solve_warp(SolveArgs a)
 {
     warp_lanes<WarpSolver<L, FAM, MIXED>, L, MIXED>(a);
 }
