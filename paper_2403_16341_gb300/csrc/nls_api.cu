@@ -111,7 +111,7 @@ struct nls_batch {
     std::map<int64_t, HostReq> hreqs;
     // cached executable graphs by request-shape signature
     std::map<std::string, cudaGraphExec_t> graphs;
-    std::map<const void *, int> occ_cache;
+    std::map<std::pair<const void *, int>, int> occ_cache; // by kernel and shared memory
     std::map<long long, Tuned> tuned;
     double *d_tune = nullptr; // autotuner scratch for a prefix of u
     size_t tune_bytes = 0;
@@ -241,14 +241,15 @@ static int select_kernel(nls_batch *h, int family, int n, int alg, KernelInfo *o
 
 static int occupancy(nls_batch *h, const KernelInfo &k, int *occ)
 {
-    auto it = h->occ_cache.find(k.func);
+    const auto key = std::make_pair(k.func, k.smem);
+    auto it = h->occ_cache.find(key);
     if (it != h->occ_cache.end()) {
         *occ = it->second;
         return NLS_OK;
     }
     int o = 0;
     NLS_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k.func, k.block, k.smem));
-    h->occ_cache[k.func] = o;
+    h->occ_cache[key] = o;
     *occ = o;
     return NLS_OK;
 }

@@ -1,0 +1,38 @@
+// nls_cols_kernels.cuh -- launch helpers and registry entries of the
+// shared-memory column solver (nls_cols.cuh): one instance per CTA, n <= 128;
+// the block and the shared memory follow n.
+#pragma once
+
+#include "nls_cols.cuh"
+#include "nls_internal.h"
+
+namespace nls {
+
+template <int FAM, bool MIXED>
+static cudaError_t launch_cols(const SolveArgs &a, int grid, cudaStream_t st)
+{
+    constexpr int C = col_panel<MIXED>();
+    k_solve_cols<C, FAM, MIXED><<<grid, 32 * col_warps<MIXED>(a.n), col_smem_bytes<C, MIXED>(a.n), st>>>(a);
+    return cudaGetLastError();
+}
+
+template <int FAM, bool MIXED>
+static KernelInfo cols_info(int n)
+{
+    if (n < 1 || n > COL_NMAX) return KernelInfo{};
+    constexpr int C = col_panel<MIXED>();
+    const void *f = reinterpret_cast<const void *>(&k_solve_cols<C, FAM, MIXED>);
+    // more than 48 KB of dynamic shared memory needs an opt-in, once per kernel
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, col_smem_bytes<C, MIXED>(COL_NMAX));
+    (void)attr;
+    KernelInfo k;
+    k.launch = &launch_cols<FAM, MIXED>;
+    k.func = f;
+    k.block = 32 * col_warps<MIXED>(n);
+    k.smem = col_smem_bytes<C, MIXED>(n);
+    k.per_cta = 1;
+    return k;
+}
+
+} // namespace nls

@@ -143,6 +143,14 @@ NLS_DI uint64_t max_mag_bits(const double (&v)[N])
 
 NLS_DI double bits_to_double(uint64_t b) { return __longlong_as_double((long long)b); }
 
+// 1/x in FP32 by the hardware approximation (relative error below 2^-23,
+// subnormals flushed).
+NLS_DI float pivot_rcp(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
 NLS_DI double rcp(double x) { return __drcp_rn(x); }
 NLS_DI float rcp(float x) { return __frcp_rn(x); }
 NLS_DI double nls_sqrt(double x) { return __dsqrt_rn(x); }

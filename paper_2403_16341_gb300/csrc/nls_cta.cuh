@@ -19,9 +19,9 @@
 // pivot rows are compacted into one tile slot, which the later steps skip.
 // The right-hand side is eliminated alongside; back substitution walks the
 // positions down.
-// This tiling serves the FP64 Newton-family solves (mixed precision takes the
-// column-panel kernel of nls_panel.cuh), and the NEXT-4 solvers and the
-// adjoint in both precisions.
+// This tiling serves the two-solve and quasi-Newton solvers (nls_cta_ext.cuh)
+// in both precisions and the adjoint; the Newton-family solves run on
+// nls_cols.cuh.
 //
 // The Jacobian tile comes from forward-mode duals over the stencil of each
 // owned row (Sec. 2.4).  The globalisations are those of the other tilings.
@@ -566,169 +566,6 @@ struct CtaSolver {
         if (status == ST_RUNNING && A.maxiters <= 0) status = ST_MAXITERS;
     }
 
-    NLS_DI void pass(const SolveArgs &A, SM &sm)
-    {
-        ++it;
-        if (need_jac) {
-            P a[R][R];
-            jacobian_tile(a, sm);
-            if (tid < n) sm.Fp[tid] = P(sm.F[tid]);
-            __syncthreads();
-            if (A.alg == ALG_TRUST_DOGLEG) {
-                ++ngrad;
-                // g = J^T F and J g
-#pragma unroll
-                for (int bb = 0; bb < R; ++bb) {
-                    P s = P(0);
-#pragma unroll
-                    for (int aa = 0; aa < R; ++aa)
-                        if (row(aa) < n) s = fma(a[aa][bb], sm.Fp[row(aa)], s);
-                    if (col(bb) < CTA_NMAX) sm.red[ty][col(bb)] = s;
-                }
-                __syncthreads();
-                if (tid < n) {
-                    P s = P(0);
-#pragma unroll
-                    for (int q = 0; q < CTA_T; ++q) s += sm.red[q][tid];
-                    sm.g[tid] = s;
-                }
-                __syncthreads();
-#pragma unroll
-                for (int aa = 0; aa < R; ++aa) {
-                    P s = P(0);
-#pragma unroll
-                    for (int bb = 0; bb < R; ++bb)
-                        if (col(bb) < n) s = fma(a[aa][bb], sm.g[col(bb)], s);
-                    sm.red[tx][row(aa)] = s;
-                }
-                __syncthreads();
-                if (tid < n) {
-                    P s = P(0);
-#pragma unroll
-                    for (int q = 0; q < CTA_T; ++q) s += sm.red[q][tid];
-                    sm.Jg[tid] = s;
-                }
-            }
-            if (tid < n) sm.rhs[tid] = -sm.Fp[tid];
-            __syncthreads();
-            const bool ok = lu_solve(a, sm);
-            if (!ok) {
-                status = ST_SINGULAR;
-                return;
-            }
-            if (tid < n) sm.dN[tid] = double(sm.x[tid]);
-            __syncthreads();
-            need_jac = false;
-        }
-        const int t = tid;
-        const bool own = t < n;
-        if (A.alg == ALG_NEWTON) {
-            if (own) sm.u[t] += sm.dN[t];
-            __syncthreads();
-            const double f = residual_t(sm.u);
-            __syncthreads();
-            if (own) sm.F[t] = f;
-            ++nfev;
-            need_jac = true;
-            set_status_from(bmax(mag_bits(f), sm), A);
-        } else if (A.alg == ALG_NEWTON_BACKTRACK) {
-            // slope F^T J dN of Eq. 9 by linearity: J dN = -F, so it is -||F||^2
-            const double s = -fF;
-            const double phi0 = 0.5 * fF;
-            double alpha = 1.0;
-            bool ok = false;
-            double f = 0.0, fFt = 0.0;
-            for (int m = 0; m < LS_MAX_TRIALS; ++m) {
-                if (own) sm.ut[t] = fma(alpha, sm.dN[t], sm.u[t]);
-                __syncthreads();
-                f = residual_t(sm.ut);
-                ++nfev;
-                fFt = f * f;
-                uint64_t mx = mag_bits(f);
-                bsum_max(fFt, mx, sm);
-                if (mx < INF64_BITS && 0.5 * fFt <= phi0 + LS_C1 * alpha * s) {
-                    ok = true;
-                    if (own) {
-                        sm.u[t] = sm.ut[t];
-                        sm.F[t] = f;
-                    }
-                    fF = fFt;
-                    __syncthreads();
-                    set_status_from(mx, A);
-                    break;
-                }
-                alpha *= LS_RHO;
-            }
-            if (!ok) {
-                status = ST_LS_FAILED;
-                return;
-            }
-            need_jac = true;
-        } else {
-            const double dn = own ? sm.dN[t] : 0.0;
-            const P gt = own ? sm.g[t] : P(0), jgt = own ? sm.Jg[t] : P(0);
-            const P D2 = P(Delta * Delta);
-            double r3[3] = {double(P(dn) * P(dn)), double(gt * gt), double(jgt * jgt)};
-            bsumk<3>(r3, sm);
-            const P nN2 = P(r3[0]), gg = P(r3[1]), JgJg = P(r3[2]);
-            const P tt = gg / JgJg;
-            const P cc = tt * tt * gg;
-            const P w = P(dn) + tt * gt;
-            // the interpolation's quadratic, only when the CTA takes branch D
-            // (a block-uniform decision, so the barriers inside are safe)
-            P aa = P(0), bb = P(0);
-            if (!(nN2 <= D2) && !(cc >= D2)) {
-                double r2[2] = {double(w * w), double(-tt * gt * w)};
-                bsumk<2>(r2, sm);
-                aa = P(r2[0]);
-                bb = P(r2[1]);
-            }
-            // pred = -2 F.Jd - ||Jd||^2 (Eq. 15) from block-uniform scalars:
-            // J dN = -F and F.(J g) = g.g (g = J^T F), so no J d is formed
-            double d, pred;
-            if (nN2 <= D2) {
-                d = dn;
-                pred = fF;
-            } else if (cc >= D2) {
-                const P sc = P(Delta) / nls_sqrt(gg);
-                d = double(-sc * gt);
-                pred = double(sc * (P(2) * gg - sc * JgJg));
-            } else {
-                const P q = cc - D2;
-                const P tau = (-bb + nls_sqrt(bb * bb - aa * q)) / aa;
-                d = double(fma(tau, w, -tt * gt));
-                const P s1 = (P(1) - tau) * tt; // J d = -s1 J g - tau F
-                pred = double(s1 * (P(2) * (P(1) - tau) * gg - s1 * JgJg) + tau * (P(2) - tau) * P(fF));
-            }
-            if (!own) d = 0.0;
-            if (own) sm.ut[t] = sm.u[t] + d;
-            __syncthreads();
-            const double f = residual_t(sm.ut);
-            ++nfev;
-            double fFt = f * f;
-            uint64_t mx = mag_bits(f);
-            bsum_max(fFt, mx, sm);
-            const double ared = fF - fFt;
-            if (tr_step_outcome(A.tr_scheme, pred > 0.0 && mx < INF64_BITS, ared, pred, !(nN2 <= D2), Delta)) {
-                if (own) {
-                    sm.u[t] = sm.ut[t];
-                    sm.F[t] = f;
-                }
-                fF = fFt;
-                need_jac = true;
-                rej = 0;
-                __syncthreads();
-                set_status_from(mx, A);
-            } else {
-                if (++rej >= TR_MAX_REJECTIONS) {
-                    status = ST_TR_STALLED;
-                    return;
-                }
-                if (it >= A.maxiters) status = ST_MAXITERS;
-            }
-        }
-    }
-
     NLS_DI void finish(const SolveArgs &A, SM &sm) const
     {
         __syncthreads();
@@ -800,12 +637,6 @@ NLS_DI void cta_loop(SolveArgs &a)
         }
         s.finish(a, sm);
     }
-}
-
-template <int R, int FAM, bool MIXED>
-__global__ void __launch_bounds__(CTA_TPB) k_solve_cta(SolveArgs a)
-{
-    cta_loop<CtaSolver<R, FAM, MIXED>>(a);
 }
 
 } // namespace nls

@@ -86,12 +86,20 @@ KernelInfo cta_ext_kernel(int family, int n, int alg, bool mixed)
 KernelInfo warp_kernel_fp64(int family, int L);
 KernelInfo warp_kernel_mixed(int family, int L);
 
-KernelInfo cta_kernel_fp64(int family, int n);
-KernelInfo cta_kernel_mixed(int family, int n);
+KernelInfo cols_kernel_cubic(int n, bool mixed);
+KernelInfo cols_kernel_bratu(int n, bool mixed);
+KernelInfo cols_kernel_square(int n, bool mixed);
+KernelInfo cols_kernel_rosenbrock(int n, bool mixed);
 
 KernelInfo cta_kernel(int family, int n, bool mixed)
 {
-    return mixed ? cta_kernel_mixed(family, n) : cta_kernel_fp64(family, n);
+    switch (family) {
+    case FAM_CUBIC: return cols_kernel_cubic(n, mixed);
+    case FAM_BRATU: return cols_kernel_bratu(n, mixed);
+    case FAM_SQUARE: return cols_kernel_square(n, mixed);
+    case FAM_ROSENBROCK: return cols_kernel_rosenbrock(n, mixed);
+    default: return KernelInfo{};
+    }
 }
 
 KernelInfo warp_kernel(int family, int n, bool mixed, int lanes)
