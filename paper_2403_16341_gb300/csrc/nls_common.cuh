@@ -151,7 +151,39 @@ NLS_DI float pivot_rcp(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-NLS_DI double rcp(double x) { return __drcp_rn(x); }
+// 1/x, correctly rounded, on the integer pipes.  Newton's method in integers:
+// with x = m 2^(e-52), m in [2^52, 2^53), a 24-bit reciprocal Y 2^-76 of m has
+// the error E = 2^76 - m Y (below 2^55, so exact in 64-bit wrap-around
+// arithmetic), and 2^106 / m = Y 2^30 / (1 - E 2^-76) is its series to second
+// order within -1 .. 2 units (checked over 10^8 mantissas); the exact
+// remainder 2^106 - q m then gives the floor, whose last bit rounds (a tie
+// would need an odd q dividing a power of two).  The FP64 unit, which takes 64
+// to 76 cycles per warp instruction and would be held for five of them, stays
+// free.  Zero, subnormal, infinite and NaN x and subnormal results take the
+// library's reciprocal.
+NLS_DI double rcp(double x)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(x);
+    const uint32_t ex = (uint32_t)(b >> 52) & 0x7ffu;
+    if (ex - 1u >= 2044u) return __drcp_rn(x);
+    const uint64_t m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    const float y = pivot_rcp(__uint_as_float(0x3f800000u | (uint32_t)((m >> 29) & 0x7fffffu))); // (1/2, 1]
+    const uint32_t Y = __float2uint_rz(y * 16777216.0f);
+    const int64_t E = -(int64_t)(m * Y);
+    const int32_t Eh = (int32_t)(E >> 32);
+    const int64_t s1 = (int64_t)(int32_t)Y * Eh + (int64_t)(((uint64_t)Y * (uint32_t)E) >> 32);
+    const uint64_t s2 = ((uint64_t)Y * (uint32_t)(((int64_t)Eh * Eh) >> 20)) >> 38;
+    uint64_t q = ((uint64_t)Y << 30) + (uint64_t)(s1 >> 14) + s2 - 1;
+    int64_t r = -(int64_t)(q * m);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+        if (r >= (int64_t)m) {
+            ++q;
+            r -= (int64_t)m;
+        }
+    const uint64_t mant = (q + 1) >> 1; // in [2^52, 2^53]: 2^53 carries into the exponent
+    return __longlong_as_double((long long)((b & 0x8000000000000000ull) | (((uint64_t)(2044u - ex) << 52) + mant)));
+}
 NLS_DI float rcp(float x) { return __frcp_rn(x); }
 NLS_DI double nls_sqrt(double x) { return __dsqrt_rn(x); }
 NLS_DI float nls_sqrt(float x) { return __fsqrt_rn(x); }
