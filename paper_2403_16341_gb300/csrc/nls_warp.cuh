@@ -269,18 +269,26 @@ struct WarpSolver {
         }
     }
 
-    // The lane of this lane's segment that holds the pivot: the largest
-    // magnitude m among the candidates, the lowest position among equals (a NaN
-    // not yet at its own pivot position was given m = 0).  All lanes call it.
-    NLS_DI int pivot_lane(K m, bool cand, int pos) const
+    // The lane of this lane's segment that holds the pivot of step k: the
+    // largest |a| among the rows left (those at positions >= k), the lowest
+    // position among equals; a NaN not at position k is never chosen.  One
+    // holder of the largest high word decides; equals, infinities and NaN take
+    // the full comparison.  All lanes call it.
+    NLS_DI int pivot_lane(P a, int k, int pos, bool left) const
     {
         const unsigned FULL = 0xffffffffu;
         const unsigned seg = L == 32 ? FULL : ((1u << (L & 31)) - 1u) << lane0;
-        const uint32_t kh = cand ? (uint32_t)(sizeof(K) == 8 ? (uint64_t)m >> 32 : (uint64_t)m) + 1u : 0u;
+        const K inf = inf_bits(P(0));
+        K m = mag_bits(a);
+        const uint32_t inf_word = sizeof(K) == 8 ? (uint32_t)((uint64_t)inf >> 32) : (uint32_t)inf;
+        const uint32_t kh = left ? (uint32_t)(sizeof(K) == 8 ? (uint64_t)m >> 32 : (uint64_t)m) + 1u : 0u;
         const uint32_t h = seg_top<L>(kh); // every lane, candidate or not
-        bool top = cand && kh == h;
-        unsigned b = __ballot_sync(FULL, top) & seg;
-        if (__any_sync(FULL, (b & (b - 1u)) != 0u)) { // several holders of the largest word
+        unsigned b = __ballot_sync(FULL, kh == h) & seg;
+        if (__any_sync(FULL, (b & (b - 1u)) != 0u || h > inf_word)) {
+            if (pos > k && m > inf) m = K(0);
+            const uint32_t gh = left ? (uint32_t)(sizeof(K) == 8 ? (uint64_t)m >> 32 : (uint64_t)m) + 1u : 0u;
+            const uint32_t g = seg_top<L>(gh);
+            bool top = left && gh == g;
             if constexpr (sizeof(K) == 8) {
                 const uint32_t kl = top ? (uint32_t)m : 0u;
                 const uint32_t l = seg_top<L>(kl);
@@ -296,15 +304,16 @@ struct WarpSolver {
     // One step of the LU at column k.  a[0] is column k of the lane's row and
     // a[c] column k + c; m = n - 1 - k columns follow the pivot.  The updated
     // column k + c goes to a[c - S]: S = 1 moves the row one column to the left.
-    template <int S, int W>
-    NLS_DI void lu_step(P *a, P &b, int k, int m, int &pos, bool &left, P &y, P &rk, bool &ok, SM &sm) const
+    // Whole chunks of columns are skipped past n: FP32 eight at a time (fewer
+    // tests), FP64 one pair.
+    template <int S, int W, class SMT>
+    NLS_DI void lu_step(P *a, P &b, int k, int m, int &pos, bool &left, P &y, P &rk, bool &ok, SMT &sm) const
     {
+        constexpr int SKIP = VEC == 4 ? 8 : 2;
         const unsigned FULL = 0xffffffffu;
         const K inf = inf_bits(P(0));
         const int lane = lane0 + r;
-        K mag = mag_bits(a[0]);
-        if (pos > k && mag > inf) mag = K(0);
-        const int src = pivot_lane(mag, left, pos);
+        const int src = pivot_lane(a[0], k, pos, left);
         const int ppos = __shfl_sync(FULL, pos, src);
         P *const row = sm.U[k];
         if (lane == src) {
@@ -312,7 +321,7 @@ struct WarpSolver {
             else *reinterpret_cast<double2 *>(row) = make_double2(b, a[0]);
 #pragma unroll
             for (int c = 1; c < W; c += VEC) {
-                if (c > m) break;
+                if ((c - 1) % SKIP == 0 && c > m) break;
                 if constexpr (VEC == 4)
                     *reinterpret_cast<float4 *>(row + 3 + c) =
                         make_float4(a[c], c + 1 < W ? a[c + 1 < W ? c + 1 : 0] : P(0),
@@ -349,7 +358,7 @@ struct WarpSolver {
         const P l = left ? a[0] * pr : P(0);
 #pragma unroll
         for (int c = 1; c < W; c += VEC) {
-            if (c > m) break;
+            if ((c - 1) % SKIP == 0 && c > m) break;
             if constexpr (VEC == 4) {
                 const float4 v = *reinterpret_cast<const float4 *>(row + 3 + c);
                 a[c - S] = a[c] - l * v.x;
@@ -377,7 +386,8 @@ struct WarpSolver {
     // for the pivot and unskipped columns: 2^16 mixed n = 32 systems
     // (backtracking) 5.66 -> 3.31 ms, 20,011 FP64 n = 27 ones 6.61 -> 5.98 ms,
     // 1,024 ten-dimensional Rosenbrock ones (trust region) 2.44 -> 1.77 ms.
-    NLS_DI bool lu_solve(P (&a)[L], P &b, SM &sm) const
+    template <class SMT>
+    NLS_DI bool lu_solve(P (&a)[L], P &b, SMT &sm) const
     {
         const unsigned FULL = 0xffffffffu;
         int pos = r;              // position of this lane's row after the interchanges
