@@ -5,9 +5,8 @@
 // return dL/dtheta = -mu^T dF/dtheta.  The Jacobian, the transpose and the
 // solve reuse the solver tilings, in FP64:
 //   * warp tiling (n <= 32): one instance per segment of L lanes; lane r
-//     builds row r of J by forward-mode duals, the segment transposes it
-//     through shared memory (lane r then holds row r of J^T) and runs the
-//     solver's LU with partial pivoting on it;
+//     builds row r of J^T (column r of J, by forward-mode duals) and the segment
+//     runs the solver's LU with partial pivoting on it;
 //   * CTA tiling (n <= 128): one instance per 256-thread CTA; the R x R
 //     register tiles of J are transposed through the CTA's shared-memory
 //     factor buffer and factored by the solver's block-cyclic LU.
@@ -36,11 +35,15 @@ struct AdjointTileArgs {
 
 // ---------------------------------------------------------------- warp
 
+// Lane r loads column r of J, i.e. row r of J^T, directly (the cubic's A by
+// columns, the stencil families' three partials from the neighbouring lanes);
+// no residual is formed and A is not kept, so a segment needs the LU's rows in
+// shared memory only and ten CTAs share an SM.
 template <int L, int FAM>
 __global__ void __launch_bounds__(WARP_TPB) k_adjoint_warp(AdjointTileArgs g)
 {
     using S = WarpSolver<L, FAM, false>;
-    using SM = typename S::SM;
+    using SM = WarpSmem<L, false, FAM_SQUARE>; // without A
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int SEGS = 32 / L;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -56,24 +59,29 @@ __global__ void __launch_bounds__(WARP_TPB) k_adjoint_warp(AdjointTileArgs g)
     s.r = lane % L;
     s.n = g.n;
     s.lane0 = seg * L;
-    SolveArgs a{};
-    a.params = g.params;
-    a.u = const_cast<double *>(g.u);
-    a.batch = B;
-    a.ld = B;
-    a.n = g.n;
-    a.maxiters = 1;
-    s.init(a, k, sm, FULL); // parameters and the root; its residual is not used
+    const bool live = s.row_live();
     double row[L];
-    s.jacobian_row(row, sm);
-    // transpose: lane r takes column r of J, i.e. row r of J^T
+    if constexpr (FAM == FAM_CUBIC) {
 #pragma unroll
-    for (int j = 0; j < L; ++j) sm.tr[s.r][j] = row[j];
-    __syncwarp();
+        for (int i = 0; i < L; ++i)
+            row[i] = (i < g.n && live) ? __ldg(g.params + (int64_t)(i * g.n + s.r) * B + k) : 0.0;
+    }
+    s.b_r = FAM == FAM_BRATU ? __ldg(g.params + k) : 0.0;
+    s.u = live ? g.u[(int64_t)s.r * B + k] : 0.0;
+    double mu = live ? g.w[(int64_t)s.r * B + k] : 0.0;
+    double d0, d1, d2;
+    s.stencil(d0, d1, d2);
+    if constexpr (FAM == FAM_CUBIC) {
 #pragma unroll
-    for (int j = 0; j < L; ++j) row[j] = sm.tr[j][s.r];
-    __syncwarp();
-    double mu = s.row_live() ? g.w[(int64_t)s.r * B + k] : 0.0;
+        for (int i = 0; i < L; ++i)
+            if (i == s.r && live) row[i] += d1;
+    } else {
+        // column r: dF_{r-1}/du_r, dF_r/du_r, dF_{r+1}/du_r
+        const double up = __shfl_up_sync(FULL, d2, 1, L), dn = __shfl_down_sync(FULL, d0, 1, L);
+#pragma unroll
+        for (int i = 0; i < L; ++i)
+            row[i] = !live ? 0.0 : i == s.r ? d1 : i == s.r - 1 ? up : (i == s.r + 1 && i < g.n) ? dn : 0.0;
+    }
     const bool ok = s.lu_solve(row, mu, sm); // mu_r = (J^-T w)_r in lane r
     const int n = g.n;
     if constexpr (FAM == FAM_CUBIC) {
@@ -100,7 +108,7 @@ static cudaError_t launch_adjoint_warp_lf(const AdjointTileArgs &g, cudaStream_t
 {
     constexpr int per_cta = (WARP_TPB / 32) * (32 / L);
     const int64_t grid = (g.batch + per_cta - 1) / per_cta;
-    k_adjoint_warp<L, FAM><<<(unsigned)grid, WARP_TPB, warp_smem_bytes<L, false, FAM>(), st>>>(g);
+    k_adjoint_warp<L, FAM><<<(unsigned)grid, WARP_TPB, warp_smem_bytes<L, false, FAM_SQUARE>(), st>>>(g);
     return cudaGetLastError();
 }
 
