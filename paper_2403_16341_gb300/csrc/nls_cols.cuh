@@ -47,7 +47,11 @@
 namespace nls {
 
 constexpr int COL_NMAX = 128;
-constexpr int COL_CHUNK = 16; // columns that a warp updates at a time
+// Columns that a warp updates at a time: one per lane of the U12 solve in mixed
+// precision, where that solve is a fifth of the instructions; FP64 16, which
+// spreads the FP64 work more evenly over the warps.
+template <bool MIXED>
+constexpr int col_chunk() { return MIXED ? 32 : 16; }
 
 // The multipliers' reciprocal pivot: in FP32 the hardware approximation
 // (pivot_rcp: its error is inside the FP32 LU's own rounding; a zero or
@@ -102,7 +106,7 @@ constexpr int col_smem_bytes(int n)
 {
     using SM = ColSmem<C, MIXED>;
     return (int)((sizeof(SM) + 15) / 16 * 16) +
-           (col_warps<MIXED>(n) * COL_CHUNK * SM::US + (n + 1) * col_ld(n)) * (MIXED ? 4 : 8);
+           (col_warps<MIXED>(n) * col_chunk<MIXED>() * SM::US + (n + 1) * col_ld(n)) * (MIXED ? 4 : 8);
 }
 
 template <int C, int FAM, bool MIXED>
@@ -111,6 +115,7 @@ struct ColSolver {
     using K = decltype(mag_bits(P(0)));
     using SM = ColSmem<C, MIXED>;
     static constexpr int US = SM::US;
+    static constexpr int CHUNK = col_chunk<MIXED>();
 
     int tid, lane, warp, nw, n, ld;
     P *A;  // the matrix, by columns; column n is the right-hand side
@@ -594,7 +599,7 @@ struct ColSolver {
         __syncwarp();
     }
 
-    // Columns j0 .. j0 + nj - 1 (nj <= COL_CHUNK) of the trailing matrix under
+    // Columns j0 .. j0 + nj - 1 (nj <= CHUNK) of the trailing matrix under
     // the panel at k0: l are this lane's rows' multipliers, pos their new
     // positions.
     template <int SK>
@@ -683,6 +688,15 @@ struct ColSolver {
     NLS_DI void trailing(int k0, int kc, int p, bool ahead, SM &sm) const
     {
         const int par = p & 1;
+        const int k1 = k0 + kc, kn = min(C, n - k1); // the next panel
+        // the columns right of the next panel, the right-hand side last
+        auto draw = [&]() {
+            int q = 0;
+            if (lane == 0) q = atomicAdd(&sm.chunk[par], 1);
+            return k1 + kn + __shfl_sync(0xffffffffu, q, 0) * CHUNK;
+        };
+        int j = ahead ? k1 : draw();
+        if (j > n) return;
         P l[SK][C];
         int pos[SK];
 #pragma unroll
@@ -694,19 +708,11 @@ struct ColSolver {
 #pragma unroll
             for (int c = 0; c < C; ++c) l[s][c] = c < q ? A[(k0 + c) * ld + pos[s]] : P(0);
         }
-        const int k1 = k0 + kc, kn = min(C, n - k1); // the next panel
         for (;;) {
-            int j = k1, nj = kn;
-            if (!ahead) { // the columns right of the next panel, the right-hand side last
-                int q = 0;
-                if (lane == 0) q = atomicAdd(&sm.chunk[par], 1);
-                q = __shfl_sync(0xffffffffu, q, 0);
-                j = k1 + kn + q * COL_CHUNK;
-                if (j > n) break;
-                nj = min(COL_CHUNK, n + 1 - j);
-            }
-            update_chunk<SK>(k0, kc, par, j, nj, l, pos, sm);
+            update_chunk<SK>(k0, kc, par, j, ahead ? kn : min(CHUNK, n + 1 - j), l, pos, sm);
             if (ahead) break;
+            j = draw();
+            if (j > n) break;
         }
     }
     NLS_DI void factor_next(int k0, int kc, int p, SM &sm) const
@@ -1025,7 +1031,7 @@ __global__ void __launch_bounds__((col_max_threads<MIXED>()), (col_min_ctas<FAM,
     s.nw = col_warps<MIXED>(a.n);
     s.ld = col_ld(a.n);
     s.A = reinterpret_cast<P *>(smem_raw + (sizeof(SM) + 15) / 16 * 16);
-    s.ub = s.A + (a.n + 1) * s.ld + s.warp * (COL_CHUNK * SM::US);
+    s.ub = s.A + (a.n + 1) * s.ld + s.warp * (Solver::CHUNK * SM::US);
     s.B = a.ld;
     s.params = a.params;
     const unsigned long long t_end = a.budget_ns ? global_ns() + a.budget_ns : ~0ull;
