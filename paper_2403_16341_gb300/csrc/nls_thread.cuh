@@ -525,7 +525,9 @@ NLS_DI void thread_lanes(SolveArgs &a)
                              k0 + THREAD_TPB <= a.batch;
             if (vec) {
                 const int half = lane >> 4, pair = 2 * (lane & 15);
-#pragma unroll 4
+                // 12 loads in flight: four left the warp waiting for nine round
+                // trips to memory per refill (n = 8), two warps share a scheduler
+#pragma unroll 12
                 for (int e0 = 0; e0 < E; e0 += 2) {
                     const int e = e0 + half;
                     if (e < E) {
@@ -542,7 +544,7 @@ NLS_DI void thread_lanes(SolveArgs &a)
             if (want && cand < a.batch) {
                 k = cand;
                 if (!vec) {
-#pragma unroll 4
+#pragma unroll 24
                     for (int e = 0; e < E; ++e) {
                         const double v = __ldg(a.params + (int64_t)e * a.ld + k);
                         sd[e * THREAD_TPB + lane] = v;
