@@ -176,7 +176,7 @@ int nls_batch_create(nls_handle *out, int device, void *cuda_stream, size_t mem_
  * returned iterate; out: optional per-instance outputs (NULL = none).
  * alg = nls_alg | nls_flags.  abstol >= 0 (finite), maxiters >= 0.
  * Requests are grouped until nls_flush or nls_status, which launch every
- * pending request of the handle together in one CUDA-graph launch: a lone
+ * pending request of the handle together (several in one CUDA-graph launch): a lone
  * request as a persistent kernel (work counter, idle lanes refilled), several
  * requests as concurrent kernel nodes with full grids whose blocks the
  * hardware interleaves.  *req receives an id for nls_status.
@@ -265,24 +265,28 @@ enum nls_option {
                                  0: one CTA per block of instances             */
     NLS_OPT_REFILL_BELOW = 2, /* thread tiling, persistent: a warp refills its
                                  idle lanes when at most this many lanes are
-                                 still iterating (0..31, default 24)           */
+                                 still iterating (0..31; unset: 24 for
+                                 NLS_ROSENBROCK, whose pass counts spread
+                                 widely, 8 for the other families)             */
     NLS_OPT_CTAS_PER_SM = 3,  /* cap on resident CTAs per SM (0 = occupancy)   */
     NLS_OPT_DEADLINE_US = 5,  /* > 0: each launch stops iterating this many
                                  microseconds (device clock) after it starts;
                                  unfinished instances end NLS_ABORTED.  0 (the
                                  default): no deadline.  Applies to requests
                                  enqueued afterwards.                          */
-    NLS_OPT_GRAPH = 4         /* 1 (default): a flush is one CUDA-graph launch
-                                 (counter reset, one kernel node per request,
-                                 all concurrent, counter read-back), cached by
-                                 the shape of the group; 0: direct launches    */
+    NLS_OPT_GRAPH = 4         /* 1 (default): a flush of several requests is one
+                                 CUDA-graph launch (one kernel node per
+                                 request, all concurrent, counter read-back),
+                                 cached by the shape of the group, a flush of
+                                 one request a kernel and a copy; 0: direct
+                                 launches                                     */
 };
 /* Errors: NLS_E_INVALID for an unknown option or a value out of range. */
 int nls_set_option(nls_handle h, int option, int64_t value);
 
 /* Autotuner: times each tiling that can hold n -- thread (n <= 8), warp with
  * 8, 16 or 32 lanes (n <= lanes), CTA (n > 8) -- each both as a persistent
- * grid (thread tiling: refill thresholds 0/16/24/31) and as a
+ * grid (thread tiling: refill thresholds 0/8/16/24/31) and as a
  * one-block-per-chunk grid (best of three runs), on the first min(batch, 2^18) instances of this
  * batch; when the two fastest are within 5%, they are timed again,
  * alternately, on the first min(batch, 2^20) instances.  Keeps the fastest

@@ -56,7 +56,7 @@ struct Request {
 
 struct Opts {
     int persistent = 1;     // persistent grid with a work counter
-    int refill_below = 24;  // refill idle lanes when running lanes <= this
+    int refill_below = -1;  // refill idle lanes when running lanes <= this (-1: default_refill)
     int ctas_per_sm = 0;    // 0 = occupancy limit
     int graph = 1;          // flush through a cached CUDA graph
     int64_t deadline_us = 0; // per-launch iteration budget (0 = none)
@@ -312,6 +312,12 @@ static int ring_take(nls_batch *h, int count, int *start)
     return NLS_OK;
 }
 
+// Refill threshold of a request's persistent thread-tiled grid: the caller's, if set.
+static int default_refill(const nls_batch *h, int family)
+{
+    return h->opt.refill_below >= 0 ? h->opt.refill_below : nls::refill_rule(family);
+}
+
 // Launch geometry of every pending request.  A lone request runs as a
 // persistent grid (one wave of CTAs drawing instances from its work counter,
 // lanes refilled as instances finish).  When several requests are flushed
@@ -343,7 +349,7 @@ static int plan_grids(nls_batch *h, const std::vector<Request *> &rs, std::vecto
         if (h->opt.ctas_per_sm > 0) occ = std::min(occ, h->opt.ctas_per_sm);
         grids[i] = (int)std::min<int64_t>(ctas, (int64_t)std::max(occ, 1) * h->sms);
         r.args.counter = h->d_ctr + r.slot + 1;
-        r.args.refill_below = r.refill >= 0 ? r.refill : h->opt.refill_below;
+        r.args.refill_below = r.refill >= 0 ? r.refill : default_refill(h, r.family);
     }
     return NLS_OK;
 }
@@ -543,7 +549,7 @@ static int launch_poly(nls_batch *h, Request &r)
         c.resid = w.cres;
         c.solved = cnt + 1;
         c.counter = cnt + 2;
-        c.refill_below = h->opt.refill_below;
+        c.refill_below = default_refill(h, r.family);
         e = ks.launch(c, grid, st);
         if (e != cudaSuccess) return fail(h, NLS_E_CUDA, "poly stage %d: %s", sidx + 1, cudaGetErrorString(e));
         nls::PolyScatterArgs sc{B, n, cnt, w.idx, w.cu, w.cst, w.cit, w.cnf, w.cres,
@@ -669,14 +675,14 @@ static int load_tuning(nls_batch *h, const char *path)
 
 // One timed trial of a tiling on the first S instances of a request; u's
 // prefix is restored from `save` before the run.
-static int tune_trial(nls_batch *h, const SolveArgs &base, const KernelInfo &k, int refill, const double *save,
-                      int64_t save_pitch, int64_t S, unsigned long long *ctr, float *ms_out)
+static int tune_trial(nls_batch *h, const SolveArgs &base, int base_family, const KernelInfo &k, int refill,
+                      const double *save, int64_t save_pitch, int64_t S, unsigned long long *ctr, float *ms_out)
 {
     SolveArgs a = base;
     a.batch = S;
     a.solved = ctr;
     a.counter = refill == REFILL_STATIC ? nullptr : ctr + 1;
-    a.refill_below = refill >= 0 ? refill : refill == REFILL_STATIC ? 0 : h->opt.refill_below;
+    a.refill_below = refill >= 0 ? refill : refill == REFILL_STATIC ? 0 : default_refill(h, base_family);
     a.status = nullptr;
     a.iters = nullptr;
     a.resid = nullptr;
@@ -1106,14 +1112,14 @@ int nls_autotune(nls_handle h, int family, const double *params, double *u, int 
     const bool ext = (alg & NLS_ALG_MASK) >= NLS_POTRA_PTAK;
     if (ext) {
         if (n <= 8)
-            for (int r : {REFILL_STATIC, 0, 16, 24, 31}) add(NLS_TILE_THREAD, 0, r);
+            for (int r : {REFILL_STATIC, 0, 8, 16, 24, 31}) add(NLS_TILE_THREAD, 0, r);
         for (int r : {REFILL_STATIC, -1}) {
             if (n <= 16) add(NLS_TILE_WARP, 16, r);
             if (n <= 32) add(NLS_TILE_WARP, 32, r);
             if (n > 8) add(NLS_TILE_CTA, 0, r);
         }
     } else if (n <= 8) {
-        for (int r : {REFILL_STATIC, 0, 16, 24, 31}) add(NLS_TILE_THREAD, 0, r);
+        for (int r : {REFILL_STATIC, 0, 8, 16, 24, 31}) add(NLS_TILE_THREAD, 0, r);
         for (int r : {REFILL_STATIC, -1}) add(NLS_TILE_WARP, 8, r);
     }
     for (int r : {REFILL_STATIC, -1}) {
@@ -1147,7 +1153,7 @@ int nls_autotune(nls_handle h, int family, const double *params, double *u, int 
         KernelInfo k = cand_kernel(c);
         if (!k.launch) continue;
         float ms = 0.f;
-        rc = tune_trial(h, base, k, c.refill, save, SF, S, ctr, &ms);
+        rc = tune_trial(h, base, family, k, c.refill, save, SF, S, ctr, &ms);
         if (rc) return rc;
         c.rate = double(S) / (double(ms) * 1e-3);
         if (c.rate > best.rate) best = c;
@@ -1168,7 +1174,7 @@ int nls_autotune(nls_handle h, int family, const double *params, double *u, int 
                     const Tuned &c = *fin[f];
                     KernelInfo k = cand_kernel(c);
                     float ms = 0.f;
-                    rc = tune_trial(h, base, k, c.refill, save, SF, SF, ctr, &ms);
+                    rc = tune_trial(h, base, family, k, c.refill, save, SF, SF, ctr, &ms);
                     if (rc) return rc;
                     bestms[f] = std::min(bestms[f], ms);
                 }

@@ -17,6 +17,17 @@ struct KernelInfo {
     int per_cta = 0;   // instances per CTA per round (static grids)
 };
 
+// Refill threshold of a persistent thread-tiled grid when the caller set none
+// (a warp refills its idle lanes when at most this many still iterate).  A
+// refill of a few lanes costs a whole warp's initial residual, idle lanes cost
+// their share of every pass: few lanes left is the better point where pass
+// counts are close together (2^19 cubic n = 8, from 24 to 8: Newton FP64 2.58 ->
+// 2.44 ms, mixed 1.21 -> 0.98; backtracking 2.94 -> 2.62 and 1.56 -> 1.19; trust
+// region 3.43 -> 3.37 and 1.30 -> 1.27; Bratu n = 8 4 to 15%; square within 1%),
+// early refills where they spread widely (Rosenbrock n = 8, trust region: 11.6
+// ms with 24, 14.2 with 8).
+inline int refill_rule(int family) { return family == FAM_ROSENBROCK ? 24 : 8; }
+
 // One instance per thread, compile-time n in 1..8.
 KernelInfo thread_kernel(int family, int n, bool mixed, bool analytic);
 
