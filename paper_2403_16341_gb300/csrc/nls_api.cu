@@ -348,6 +348,13 @@ static int plan_grids(nls_batch *h, const std::vector<Request *> &rs, std::vecto
         if (rc) return rc;
         if (h->opt.ctas_per_sm > 0) occ = std::min(occ, h->opt.ctas_per_sm);
         grids[i] = (int)std::min<int64_t>(ctas, (int64_t)std::max(occ, 1) * h->sms);
+        if (grids[i] == ctas) {
+            // every instance has its slot in the first wave: nothing to draw from a
+            // counter (two round trips to it per warp, half of them in vain)
+            r.args.counter = nullptr;
+            r.args.refill_below = 0;
+            continue;
+        }
         r.args.counter = h->d_ctr + r.slot + 1;
         r.args.refill_below = r.refill >= 0 ? r.refill : default_refill(h, r.family);
     }
@@ -420,16 +427,27 @@ static int launch_graph(nls_batch *h, const std::vector<Request *> &rs, const st
     return NLS_OK;
 }
 
+constexpr int MIRROR_MAX_GRID = 4096;
+
 static int launch_direct(nls_batch *h, const std::vector<Request *> &rs, const std::vector<int> &grids, int s0,
-                         int nctr)
+                         int nctr, bool captured)
 {
     const cudaStream_t st = launch_stream(h);
+    // A lone request on a small grid counts its solved instances in the pinned
+    // mirror itself: one add per warp (CTA tiling: per instance) over the link
+    // instead of a copy behind the kernel.
+    const bool mirror = !captured && rs.size() == 1 && grids[0] > 0 && grids[0] <= MIRROR_MAX_GRID;
+    if (mirror) {
+        h->h_ctr[rs[0]->slot] = 0;
+        rs[0]->args.solved = h->h_ctr + rs[0]->slot;
+    }
     for (size_t i = 0; i < rs.size(); ++i) {
         if (!grids[i]) continue;
         cudaError_t e = rs[i]->kern.launch(rs[i]->args, grids[i], st);
         if (e != cudaSuccess) return fail(h, NLS_E_CUDA, "kernel launch: %s", cudaGetErrorString(e));
         ++h->launches;
     }
+    if (mirror) return NLS_OK;
     NLS_CUDA(h, cudaMemcpyAsync(h->h_ctr + s0, h->d_ctr + s0, sizeof(unsigned long long) * nctr,
                                 cudaMemcpyDeviceToHost, st));
     return NLS_OK;
@@ -612,7 +630,7 @@ static int flush_pending(nls_batch *h)
     // the host than building, updating and launching a graph of them (1,024
     // cubic n = 3 systems by Newton, the whole call: 58.5 -> 52.6 us).
     rc = h->opt.graph && nreq > 1 ? launch_graph(h, rs, grids, s0, 2 * nreq)
-                                  : launch_direct(h, rs, grids, s0, 2 * nreq);
+                                  : launch_direct(h, rs, grids, s0, 2 * nreq, cap != cudaStreamCaptureStatusNone);
     if (rc) return rc;
     bool any_poly = false;
     for (Request *r : rs)
