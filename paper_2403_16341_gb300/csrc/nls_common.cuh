@@ -141,6 +141,17 @@ NLS_DI uint64_t max_mag_bits(const double (&v)[N])
     return m;
 }
 
+// -x as an integer operation on the sign bit that the compiler does not see
+// through: a plain negation sinks into the row interchanges of the LU, where
+// it comes out as an FP64 add per pair of rows.
+NLS_DI double flip_sign(double x)
+{
+    unsigned h = (unsigned)__double2hiint(x);
+    asm("xor.b32 %0, %0, 0x80000000;" : "+r"(h));
+    return __hiloint2double((int)h, __double2loint(x));
+}
+NLS_DI float flip_sign(float x) { return -x; }
+
 NLS_DI double bits_to_double(uint64_t b) { return __longlong_as_double((long long)b); }
 
 // 1/x in FP32 by the hardware approximation (relative error below 2^-23,

@@ -335,7 +335,7 @@ struct ThreadSolver {
             // leaves the region (J is re-evaluated then: the LU overwrites it)
             have_g = false;
 #pragma unroll
-            for (int i = 0; i < N; ++i) b[i] = -Fp(i);
+            for (int i = 0; i < N; ++i) b[i] = flip_sign(Fp(i));
             if (!lu_solve<N, P>(J, b)) {
                 status = ST_SINGULAR;
                 return;
