@@ -126,7 +126,15 @@ NLS_DI void apply_dyn_batch(SolveArgs &a)
 constexpr uint64_t INF64_BITS = 0x7FF0000000000000ull;
 constexpr uint32_t INF32_BITS = 0x7F800000u;
 
-NLS_DI uint64_t mag_bits(double x) { return (uint64_t)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull; }
+// The mask is opaque to the compiler, which otherwise sees an absolute value in
+// it and forms that on the FP64 unit (a DADD): counters showed 52 of the 429
+// FP64 instructions of an n = 8 FP64 pass, and 24 of 117 of a mixed one.
+NLS_DI uint64_t mag_bits(double x)
+{
+    unsigned h = (unsigned)__double2hiint(x);
+    asm("and.b32 %0, %0, 0x7fffffff;" : "+r"(h));
+    return ((uint64_t)h << 32) | (unsigned)__double2loint(x);
+}
 NLS_DI uint32_t mag_bits(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
 NLS_DI uint64_t inf_bits(double) { return INF64_BITS; }
 NLS_DI uint32_t inf_bits(float) { return INF32_BITS; }
