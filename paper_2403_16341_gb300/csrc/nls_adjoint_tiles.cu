@@ -61,10 +61,12 @@ __global__ void __launch_bounds__(WARP_TPB) k_adjoint_warp(AdjointTileArgs g)
     s.lane0 = seg * L;
     const bool live = s.row_live();
     double row[L];
+    double diag = 0.0; // A_rr
     if constexpr (FAM == FAM_CUBIC) {
 #pragma unroll
         for (int i = 0; i < L; ++i)
             row[i] = (i < g.n && live) ? __ldg(g.params + (int64_t)(i * g.n + s.r) * B + k) : 0.0;
+        if (live) diag = __ldg(g.params + (int64_t)(s.r * g.n + s.r) * B + k);
     }
     s.b_r = FAM == FAM_BRATU ? __ldg(g.params + k) : 0.0;
     s.u = live ? g.u[(int64_t)s.r * B + k] : 0.0;
@@ -72,9 +74,10 @@ __global__ void __launch_bounds__(WARP_TPB) k_adjoint_warp(AdjointTileArgs g)
     double d0, d1, d2;
     s.stencil(d0, d1, d2);
     if constexpr (FAM == FAM_CUBIC) {
+        diag += d1; // one FP64 add, not one per row under a select
 #pragma unroll
         for (int i = 0; i < L; ++i)
-            if (i == s.r && live) row[i] += d1;
+            if (i == s.r && live) row[i] = diag;
     } else {
         // column r: dF_{r-1}/du_r, dF_r/du_r, dF_{r+1}/du_r
         const double up = __shfl_up_sync(FULL, d2, 1, L), dn = __shfl_down_sync(FULL, d0, 1, L);

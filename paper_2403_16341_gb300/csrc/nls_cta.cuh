@@ -228,7 +228,7 @@ struct CtaSolver {
                     if constexpr (FAM == FAM_CUBIC) {
                         // linear part's coefficient, plus d(u_i^3)/du_i on the diagonal
                         v = P(__ldg(params + (int64_t)(i * n + j) * B + k));
-                        if (j == i) v += d1;
+                        if (aa == bb && j == i) v += d1;
                     } else {
                         // stencil families: row i depends on u_{i-1}, u_i, u_{i+1} only
                         if (j == i - 1) v = d0;

@@ -201,13 +201,16 @@ struct WarpSolver {
     NLS_DI void jacobian_row(P (&a)[L], const SM &sm, P d0, P d1, P d2) const
     {
         if constexpr (FAM == FAM_CUBIC) {
-            // linear coefficients of F_r, then d(u_r^3)/du_r on the diagonal
+            // linear coefficients of F_r, plus d(u_r^3)/du_r on the diagonal (FP64:
+            // added once, not in every column under a select)
+            P diag = P(0);
+            if constexpr (!MIXED) diag = sm.A[r][r] + d1;
 #pragma unroll
             for (int j = 0; j < L; ++j) {
                 P v;
-                if constexpr (MIXED) v = arowf[j];
-                else v = P(sm.A[r][j]);
-                a[j] = (j < n && row_live()) ? ((j == r) ? v + d1 : v) : P(0);
+                if constexpr (MIXED) v = (j == r) ? arowf[j] + d1 : arowf[j];
+                else v = (j == r) ? diag : sm.A[r][j];
+                a[j] = (j < n && row_live()) ? v : P(0);
             }
         } else {
 #pragma unroll
@@ -307,7 +310,7 @@ struct WarpSolver {
     // Whole chunks of columns are skipped past n: FP32 eight at a time (fewer
     // tests), FP64 one pair.
     template <int S, int W, class SMT>
-    NLS_DI void lu_step(P *a, P &b, int k, int m, int &pos, bool &left, P &y, P &rk, bool &ok, SMT &sm) const
+    NLS_DI void lu_step(P *a, P &b, int k, int m, int &pos, bool &left, bool &ok, SMT &sm) const
     {
         constexpr int SKIP = VEC == 4 ? 8 : 2;
         const unsigned FULL = 0xffffffffu;
@@ -345,10 +348,7 @@ struct WarpSolver {
         const K pm = mag_bits(p0);
         if (pm == K(0) || pm >= inf) ok = false;
         const P pr = rcp(p0);
-        if (r == k) {
-            y = pb;
-            rk = pr;
-        }
+        if (r == 0) sm.vec[k] = pr;
         // the row at position k moves to the pivot's old position
         if (left && pos == k) pos = ppos;
         if (lane == src) {
@@ -392,27 +392,29 @@ struct WarpSolver {
         const unsigned FULL = 0xffffffffu;
         int pos = r;              // position of this lane's row after the interchanges
         bool left = row_live();   // not a pivot row yet
-        P y = P(0), rk = P(0);    // lane k: right-hand side and reciprocal of pivot row k
         bool ok = true;
         if constexpr (MIXED) {
-            for (int k = 0; k < n; ++k) lu_step<1, L>(a, b, k, n - 1 - k, pos, left, y, rk, ok, sm);
+            for (int k = 0; k < n; ++k) lu_step<1, L>(a, b, k, n - 1 - k, pos, left, ok, sm);
         } else {
             static_for<0, L>([&](auto Kc) {
                 constexpr int k = decltype(Kc)::value;
-                if (k < n) lu_step<0, L - k>(a + k, b, k, n - 1 - k, pos, left, y, rk, ok, sm);
+                if (k < n) lu_step<0, L - k>(a + k, b, k, n - 1 - k, pos, left, ok, sm);
             });
         }
-        // back substitution: lane k holds pivot row k's right-hand side; x_k goes
-        // to every lane, and the lanes of earlier positions remove its contribution
-        P x = P(0);
+        __syncwarp(); // the reciprocals are written
+        // back substitution: lane k takes pivot row k's right-hand side and
+        // reciprocal; x_k goes to every lane, and the lanes of earlier positions
+        // remove its contribution
+        const bool live = row_live();
+        P y = live ? sm.U[r][VEC - 2] : P(0);
+        const P rk = live ? sm.vec[r] : P(0);
 #pragma unroll 4
-        for (int k = n - 1; k >= 0; --k) {
+        for (int k = n - 1; k > 0; --k) {
             const P xk = __shfl_sync(FULL, y * rk, k, L);
-            if (r == k) x = xk;
             if (r < k) y -= sm.U[r][VEC - 1 + k - r] * xk;
         }
         __syncwarp(); // U is free for the next use
-        b = x;
+        b = y * rk;
         return ok;
     }
 
