@@ -106,7 +106,7 @@ struct nls_batch {
     std::vector<int64_t> owner;          // ring slot -> request id (0 = free)
     int ring_pos = 0;
     int ring_zeroed = 0;                 // entries [ring_pos, ring_zeroed) are free and zero
-    cudaStream_t s_zero = nullptr;       // zeroes ring blocks from the second lap on (created on first use)
+    cudaStream_t s_zero = nullptr;       // zeroes the ring, block by block from the second lap on
     // nls_solve_host / nls_solve_host_async: staging blocks not in use (by
     // size), events not in use, and the requests in flight
     std::multimap<size_t, void *> stage_free;
@@ -302,7 +302,6 @@ static int ring_take(nls_batch *h, int count, int *start)
         }
         // no launch uses these entries: a stream of its own, waited for, so that
         // the launches' streams are not
-        if (!h->s_zero) NLS_CUDA(h, cudaStreamCreateWithFlags(&h->s_zero, cudaStreamNonBlocking));
         NLS_CUDA(h, cudaMemsetAsync(h->d_ctr + z0, 0, sizeof(unsigned long long) * (z1 - z0), h->s_zero));
         NLS_CUDA(h, cudaStreamSynchronize(h->s_zero));
         h->ring_zeroed = z1;
@@ -761,11 +760,15 @@ int nls_batch_create(nls_handle *out, int device, void *cuda_stream, size_t mem_
         return fail(nullptr, NLS_E_CUDA, "cudaMallocHost: %s", cudaGetErrorString(e));
     }
     h->owner.assign(RING, 0);
-    e = cudaMemset(h->d_ctr, 0, sizeof(unsigned long long) * RING);
+    // zero before any stream of this handle or of its caller can use it
+    e = cudaStreamCreateWithFlags(&h->s_zero, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->d_ctr, 0, sizeof(unsigned long long) * RING, h->s_zero);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->s_zero);
     if (e != cudaSuccess) {
+        if (h->s_zero) cudaStreamDestroy(h->s_zero);
         cudaFree(h->d_ctr);
         cudaFreeHost(h->h_ctr);
-        return fail(nullptr, NLS_E_CUDA, "cudaMemset: %s", cudaGetErrorString(e));
+        return fail(nullptr, NLS_E_CUDA, "counter ring: %s", cudaGetErrorString(e));
     }
     h->ring_zeroed = RING;
     if (const char *cache = std::getenv("NLS_TUNE_CACHE")) load_tuning(h.get(), cache);
