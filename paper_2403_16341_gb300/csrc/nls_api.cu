@@ -105,8 +105,9 @@ struct nls_batch {
     unsigned long long *h_ctr = nullptr; // pinned mirror
     std::vector<int64_t> owner;          // ring slot -> request id (0 = free)
     int ring_pos = 0;
-    int ring_zeroed = 0;                 // entries [ring_pos, ring_zeroed) are free and zero
-    cudaStream_t s_zero = nullptr;       // zeroes the ring, block by block from the second lap on
+    int ring_zeroed = 0;                 // entries [ring_pos, ring_zeroed) are free and zero,
+    cudaStream_t zero_on = nullptr;      // by a memset on this stream,
+    cudaEvent_t zero_ev = nullptr;       // which launches on others wait for
     // nls_solve_host / nls_solve_host_async: staging blocks not in use (by
     // size), events not in use, and the requests in flight
     std::multimap<size_t, void *> stage_free;
@@ -275,18 +276,21 @@ static int wait_event(nls_batch *h, cudaEvent_t ev, int timeout_ms)
     }
 }
 
-// Reserve `count` consecutive ring entries, all zero.  Blocks of the ring are
-// zeroed as the position reaches them (once per RING_BLOCK entries, so a flush
-// needs no memset of its own); requests still owning entries of such a block
-// are waited for and their solved counts kept on the host first.
-static int ring_take(nls_batch *h, int count, int *start)
+// Reserve `count` consecutive ring entries, zero in the launch stream's order.
+// Blocks of the ring are zeroed on the launch stream as the position reaches
+// them (once per RING_BLOCK entries, so a flush needs no memset of its own);
+// requests still owning entries of such a block are waited for and their
+// solved counts kept on the host first.  What a stream capture records zeroes
+// its own entries, so a block is only taken up to them.
+static int ring_take(nls_batch *h, int count, bool captured, int *start)
 {
     if (count > RING) return fail(h, NLS_E_INVALID, "too many requests in one flush (%d)", count / 2);
     if (h->ring_pos + count > RING) h->ring_pos = h->ring_zeroed = 0;
     const int s = h->ring_pos;
+    const cudaStream_t st = launch_stream(h);
     if (s + count > h->ring_zeroed) {
         const int z0 = h->ring_zeroed;
-        const int z1 = std::min(RING, (s + count + RING_BLOCK - 1) / RING_BLOCK * RING_BLOCK);
+        const int z1 = captured ? s + count : std::min(RING, (s + count + RING_BLOCK - 1) / RING_BLOCK * RING_BLOCK);
         for (int i = z0; i < z1; ++i) {
             const int64_t id = h->owner[i];
             if (!id) continue;
@@ -300,12 +304,15 @@ static int ring_take(nls_batch *h, int count, int *start)
             }
             h->owner[i] = 0;
         }
-        // no launch uses these entries: a stream of its own, waited for, so that
-        // the launches' streams are not
-        NLS_CUDA(h, cudaMemsetAsync(h->d_ctr + z0, 0, sizeof(unsigned long long) * (z1 - z0), h->s_zero));
-        NLS_CUDA(h, cudaStreamSynchronize(h->s_zero));
+        if (!captured) {
+            if (!h->zero_ev) NLS_CUDA(h, cudaEventCreateWithFlags(&h->zero_ev, cudaEventDisableTiming));
+            NLS_CUDA(h, cudaMemsetAsync(h->d_ctr + z0, 0, sizeof(unsigned long long) * (z1 - z0), st));
+            NLS_CUDA(h, cudaEventRecord(h->zero_ev, st));
+            h->zero_on = st;
+        }
         h->ring_zeroed = z1;
     }
+    if (!captured && st != h->zero_on) NLS_CUDA(h, cudaStreamWaitEvent(st, h->zero_ev, 0));
     h->ring_pos = s + count;
     *start = s;
     return NLS_OK;
@@ -596,8 +603,12 @@ static int flush_pending(nls_batch *h)
 {
     if (h->pending.empty()) return NLS_OK;
     const int nreq = (int)h->pending.size();
+    // what a stream capture records may run many times: it zeroes its counters itself
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(launch_stream(h), &cap) != cudaSuccess) cudaGetLastError();
+    const bool captured = cap != cudaStreamCaptureStatusNone;
     int s0 = 0;
-    int rc = ring_take(h, 2 * nreq, &s0);
+    int rc = ring_take(h, 2 * nreq, captured, &s0);
     if (rc) return rc;
     cudaEvent_t done = nullptr;
     rc = take_event(h, &done);
@@ -620,16 +631,13 @@ static int flush_pending(nls_batch *h)
     std::vector<int> grids;
     rc = plan_grids(h, rs, grids);
     if (rc) return rc;
-    // what a stream capture records may run many times: it zeroes its counters itself
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(launch_stream(h), &cap) != cudaSuccess) cudaGetLastError();
-    if (cap != cudaStreamCaptureStatusNone)
+    if (captured)
         NLS_CUDA(h, cudaMemsetAsync(h->d_ctr + s0, 0, sizeof(unsigned long long) * 2 * nreq, launch_stream(h)));
     // A lone request is launched directly: one kernel and one copy cost less on
     // the host than building, updating and launching a graph of them (1,024
     // cubic n = 3 systems by Newton, the whole call: 58.5 -> 52.6 us).
     rc = h->opt.graph && nreq > 1 ? launch_graph(h, rs, grids, s0, 2 * nreq)
-                                  : launch_direct(h, rs, grids, s0, 2 * nreq, cap != cudaStreamCaptureStatusNone);
+                                  : launch_direct(h, rs, grids, s0, 2 * nreq, captured);
     if (rc) return rc;
     bool any_poly = false;
     for (Request *r : rs)
@@ -760,17 +768,6 @@ int nls_batch_create(nls_handle *out, int device, void *cuda_stream, size_t mem_
         return fail(nullptr, NLS_E_CUDA, "cudaMallocHost: %s", cudaGetErrorString(e));
     }
     h->owner.assign(RING, 0);
-    // zero before any stream of this handle or of its caller can use it
-    e = cudaStreamCreateWithFlags(&h->s_zero, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->d_ctr, 0, sizeof(unsigned long long) * RING, h->s_zero);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->s_zero);
-    if (e != cudaSuccess) {
-        if (h->s_zero) cudaStreamDestroy(h->s_zero);
-        cudaFree(h->d_ctr);
-        cudaFreeHost(h->h_ctr);
-        return fail(nullptr, NLS_E_CUDA, "counter ring: %s", cudaGetErrorString(e));
-    }
-    h->ring_zeroed = RING;
     if (const char *cache = std::getenv("NLS_TUNE_CACHE")) load_tuning(h.get(), cache);
     *out = h.release();
     return NLS_OK;
@@ -1066,7 +1063,7 @@ int nls_batch_destroy(nls_handle h)
     for (auto &kv : h->stage_free) cudaFree(kv.second);
     if (h->d_ctr) cudaFree(h->d_ctr);
     if (h->h_ctr) cudaFreeHost(h->h_ctr);
-    if (h->s_zero) cudaStreamDestroy(h->s_zero);
+    if (h->zero_ev) cudaEventDestroy(h->zero_ev);
     for (cudaEvent_t e : h->ev_free) cudaEventDestroy(e);
     if (h->s_in) cudaStreamDestroy(h->s_in);
     if (h->s_out) cudaStreamDestroy(h->s_out);
