@@ -202,13 +202,19 @@ struct WarpSolver {
     {
         if constexpr (FAM == FAM_CUBIC) {
             // linear coefficients of F_r, plus d(u_r^3)/du_r on the diagonal (FP64:
-            // added once, not in every column under a select)
+            // added once, not in every column under a select).  Mixed: added to
+            // every column (0 off the diagonal) with 32 lanes, which keeps the copy
+            // of the row in registers (2^16 n = 32 systems 3.00 -> 2.91 ms); the
+            // select, which the compiler answers with a copy in local memory and
+            // half the registers, is the better one below (uneven 2^18 mix 2.77 ->
+            // 2.71 ms)
             P diag = P(0);
             if constexpr (!MIXED) diag = sm.A[r][r] + d1;
 #pragma unroll
             for (int j = 0; j < L; ++j) {
                 P v;
-                if constexpr (MIXED) v = (j == r) ? arowf[j] + d1 : arowf[j];
+                if constexpr (MIXED && L == 32) v = arowf[j] + ((j == r) ? d1 : 0.f);
+                else if constexpr (MIXED) v = (j == r) ? arowf[j] + d1 : arowf[j];
                 else v = (j == r) ? diag : sm.A[r][j];
                 a[j] = (j < n && row_live()) ? v : P(0);
             }
@@ -275,19 +281,20 @@ struct WarpSolver {
     // The lane of this lane's segment that holds the pivot of step k: the
     // largest |a| among the rows left (those at positions >= k), the lowest
     // position among equals; a NaN not at position k is never chosen.  One
-    // holder of the largest high word decides; equals, infinities and NaN take
-    // the full comparison.  All lanes call it.
-    NLS_DI int pivot_lane(P a, int k, int pos, bool left) const
+    // holder of the largest high word decides (kh, h: this lane's word and the
+    // largest, from pivot_word); equals, infinities and NaN take the full
+    // comparison.  All lanes call it.
+    NLS_DI int pivot_lane(P a, uint32_t kh, uint32_t h, int k, int pos, bool left) const
     {
         const unsigned FULL = 0xffffffffu;
         const unsigned seg = L == 32 ? FULL : ((1u << (L & 31)) - 1u) << lane0;
         const K inf = inf_bits(P(0));
         K m = mag_bits(a);
         const uint32_t inf_word = sizeof(K) == 8 ? (uint32_t)((uint64_t)inf >> 32) : (uint32_t)inf;
-        const uint32_t kh = left ? (uint32_t)(sizeof(K) == 8 ? (uint64_t)m >> 32 : (uint64_t)m) + 1u : 0u;
-        const uint32_t h = seg_top<L>(kh); // every lane, candidate or not
         unsigned b = __ballot_sync(FULL, kh == h) & seg;
-        if (__any_sync(FULL, (b & (b - 1u)) != 0u || h > inf_word)) {
+        bool more = (b & (b - 1u)) != 0u || h > inf_word;
+        if constexpr (L < 32) more = __any_sync(FULL, more);
+        if (more) {
             if (pos > k && m > inf) m = K(0);
             const uint32_t gh = left ? (uint32_t)(sizeof(K) == 8 ? (uint64_t)m >> 32 : (uint64_t)m) + 1u : 0u;
             const uint32_t g = seg_top<L>(gh);
@@ -304,19 +311,32 @@ struct WarpSolver {
         return __ffs(b) - 1;
     }
 
+    // The magnitude's high word + 1 of a candidate (0: none) and the segment's largest.
+    NLS_DI static void pivot_word(P a, bool left, uint32_t &kh, uint32_t &h)
+    {
+        const K m = mag_bits(a);
+        kh = left ? (uint32_t)(sizeof(K) == 8 ? (uint64_t)m >> 32 : (uint64_t)m) + 1u : 0u;
+        h = seg_top<L>(kh); // every lane, candidate or not
+    }
+
     // One step of the LU at column k.  a[0] is column k of the lane's row and
     // a[c] column k + c; m = n - 1 - k columns follow the pivot.  The updated
     // column k + c goes to a[c - S]: S = 1 moves the row one column to the left.
     // Whole chunks of columns are skipped past n: FP32 eight at a time (fewer
-    // tests), FP64 one pair.
+    // tests), FP64 one pair.  In FP64 the next step's search (kh, h) starts as soon
+    // as its column is updated, so the reduction runs behind the other columns'
+    // updates (20,011 n = 27 systems: 5.18 -> 4.92 ms); the mixed loop, bound by
+    // its instructions, ran 6% slower that way in a flush of many sizes.
     template <int S, int W, class SMT>
-    NLS_DI void lu_step(P *a, P &b, int k, int m, int &pos, bool &left, bool &ok, SMT &sm) const
+    NLS_DI void lu_step(P *a, P &b, int k, int m, int &pos, bool &left, bool &ok, uint32_t &kh, uint32_t &h,
+                        SMT &sm) const
     {
         constexpr int SKIP = VEC == 4 ? 8 : 2;
         const unsigned FULL = 0xffffffffu;
         const K inf = inf_bits(P(0));
         const int lane = lane0 + r;
-        const int src = pivot_lane(a[0], k, pos, left);
+        if constexpr (VEC == 4) pivot_word(a[0], left, kh, h);
+        const int src = pivot_lane(a[0], kh, h, k, pos, left);
         const int ppos = __shfl_sync(FULL, pos, src);
         P *const row = sm.U[k];
         if (lane == src) {
@@ -368,6 +388,7 @@ struct WarpSolver {
             } else {
                 const double2 v = *reinterpret_cast<const double2 *>(row + 1 + c);
                 a[c - S] = a[c] - l * v.x;
+                if (c == 1) pivot_word(a[1 - S], left, kh, h);
                 if (c + 1 < W && c + 1 <= m) a[c + 1 - S] = a[c + 1] - l * v.y;
             }
         }
@@ -384,8 +405,8 @@ struct WarpSolver {
     // shifting loop measured 6.98 ms on 20,011 trust-region n = 27 systems).
     // Against whole rows written by scalar stores, 64-bit shuffle butterflies
     // for the pivot and unskipped columns: 2^16 mixed n = 32 systems
-    // (backtracking) 5.66 -> 3.31 ms, 20,011 FP64 n = 27 ones 6.61 -> 5.98 ms,
-    // 1,024 ten-dimensional Rosenbrock ones (trust region) 2.44 -> 1.77 ms.
+    // (backtracking) 5.66 -> 2.92 ms, 20,011 FP64 n = 27 ones (trust region) 6.61
+    // -> 4.92 ms, 1,024 ten-dimensional Rosenbrock ones 2.72 -> 1.83 ms.
     template <class SMT>
     NLS_DI bool lu_solve(P (&a)[L], P &b, SMT &sm) const
     {
@@ -393,12 +414,14 @@ struct WarpSolver {
         int pos = r;              // position of this lane's row after the interchanges
         bool left = row_live();   // not a pivot row yet
         bool ok = true;
+        uint32_t kh = 0, h = 0;
+        if constexpr (!MIXED) pivot_word(a[0], left, kh, h);
         if constexpr (MIXED) {
-            for (int k = 0; k < n; ++k) lu_step<1, L>(a, b, k, n - 1 - k, pos, left, ok, sm);
+            for (int k = 0; k < n; ++k) lu_step<1, L>(a, b, k, n - 1 - k, pos, left, ok, kh, h, sm);
         } else {
             static_for<0, L>([&](auto Kc) {
                 constexpr int k = decltype(Kc)::value;
-                if (k < n) lu_step<0, L - k>(a + k, b, k, n - 1 - k, pos, left, ok, sm);
+                if (k < n) lu_step<0, L - k>(a + k, b, k, n - 1 - k, pos, left, ok, kh, h, sm);
             });
         }
         __syncwarp(); // the reciprocals are written
