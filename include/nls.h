@@ -266,8 +266,8 @@ enum nls_option {
     NLS_OPT_REFILL_BELOW = 2, /* thread tiling, persistent: a warp refills its
                                  idle lanes when at most this many lanes are
                                  still iterating (0..31; unset: 24 for
-                                 NLS_ROSENBROCK, whose pass counts spread
-                                 widely, 8 for the other families)             */
+                                 NLS_ROSENBROCK and NLS_POTRA_PTAK, whose pass
+                                 counts spread widely, 8 otherwise)            */
     NLS_OPT_CTAS_PER_SM = 3,  /* cap on resident CTAs per SM (0 = occupancy)   */
     NLS_OPT_DEADLINE_US = 5,  /* > 0: each launch stops iterating this many
                                  microseconds (device clock) after it starts;

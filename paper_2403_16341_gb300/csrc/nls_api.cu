@@ -319,9 +319,9 @@ static int ring_take(nls_batch *h, int count, bool captured, int *start)
 }
 
 // Refill threshold of a request's persistent thread-tiled grid: the caller's, if set.
-static int default_refill(const nls_batch *h, int family)
+static int default_refill(const nls_batch *h, int family, int alg)
 {
-    return h->opt.refill_below >= 0 ? h->opt.refill_below : nls::refill_rule(family);
+    return h->opt.refill_below >= 0 ? h->opt.refill_below : nls::refill_rule(family, alg);
 }
 
 // Launch geometry of every pending request.  A lone request runs as a
@@ -362,7 +362,7 @@ static int plan_grids(nls_batch *h, const std::vector<Request *> &rs, std::vecto
             continue;
         }
         r.args.counter = h->d_ctr + r.slot + 1;
-        r.args.refill_below = r.refill >= 0 ? r.refill : default_refill(h, r.family);
+        r.args.refill_below = r.refill >= 0 ? r.refill : default_refill(h, r.family, r.args.alg);
     }
     return NLS_OK;
 }
@@ -573,7 +573,7 @@ static int launch_poly(nls_batch *h, Request &r)
         c.resid = w.cres;
         c.solved = cnt + 1;
         c.counter = cnt + 2;
-        c.refill_below = default_refill(h, r.family);
+        c.refill_below = default_refill(h, r.family, stages[sidx]);
         e = ks.launch(c, grid, st);
         if (e != cudaSuccess) return fail(h, NLS_E_CUDA, "poly stage %d: %s", sidx + 1, cudaGetErrorString(e));
         nls::PolyScatterArgs sc{B, n, cnt, w.idx, w.cu, w.cst, w.cit, w.cnf, w.cres,
@@ -707,7 +707,7 @@ static int tune_trial(nls_batch *h, const SolveArgs &base, int base_family, cons
     a.batch = S;
     a.solved = ctr;
     a.counter = refill == REFILL_STATIC ? nullptr : ctr + 1;
-    a.refill_below = refill >= 0 ? refill : refill == REFILL_STATIC ? 0 : default_refill(h, base_family);
+    a.refill_below = refill >= 0 ? refill : refill == REFILL_STATIC ? 0 : default_refill(h, base_family, base.alg);
     a.status = nullptr;
     a.iters = nullptr;
     a.resid = nullptr;

@@ -26,7 +26,9 @@ struct KernelInfo {
 // region 3.43 -> 3.37 and 1.30 -> 1.27; Bratu n = 8 4 to 15%; square within 1%),
 // early refills where they spread widely (Rosenbrock n = 8, trust region: 11.6
 // ms with 24, 14.2 with 8).
-inline int refill_rule(int family) { return family == FAM_ROSENBROCK ? 24 : 8; }
+// Potra-Ptak, a local method that can wander, keeps 24 too (mixed cubic n = 8:
+// 2.01 ms, 2.09 with 8).
+inline int refill_rule(int family, int alg) { return family == FAM_ROSENBROCK || alg == ALG_POTRA_PTAK ? 24 : 8; }
 
 // One instance per thread, compile-time n in 1..8.
 KernelInfo thread_kernel(int family, int n, bool mixed, bool analytic);

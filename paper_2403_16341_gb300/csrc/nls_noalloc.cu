@@ -135,7 +135,7 @@ extern "C" int nls_solve_noalloc(void *cuda_stream, const nls_group *groups, int
         a.ngrad = q.out.ngrad;
         a.solved = scratch + 2 * g;
         a.counter = scratch + 2 * g + 1;
-        a.refill_below = nls::refill_rule(q.family);
+        a.refill_below = nls::refill_rule(q.family, a.alg);
         int occ = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern[g].func, kern[g].block, kern[g].smem);
         if (e != cudaSuccess) return err(NLS_E_CUDA, "occupancy query: %s", cudaGetErrorString(e));

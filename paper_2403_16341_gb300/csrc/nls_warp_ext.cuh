@@ -354,8 +354,19 @@ struct warp_ext_solver<L, FAM, MIXED, ALG_BROYDEN> {
     using type = WarpSolverBroyden<L, FAM, MIXED>;
 };
 
+// CTAs per SM that the compiler makes room for (0: its own choice).  Left alone,
+// the mixed 32-lane Bratu kernels took 205 (Broyden) and 143 registers (two-solve)
+// where 128-thread CTAs had kept them at 167 and 119: ten and fourteen warps per
+// SM instead of twelve and sixteen (2^15 Bratu n = 32 systems: modified Broyden
+// 3.30 ms against 2.66, Potra-Ptak 1.08 against 1.01).
 template <int L, int FAM, bool MIXED, int ALG>
-__global__ void __launch_bounds__(WARP_TPB) k_solve_warp_ext(SolveArgs a)
+constexpr int warp_ext_min_ctas()
+{
+    return L == 32 && MIXED && FAM == FAM_BRATU ? (ALG == ALG_BROYDEN ? 6 : 8) : 0;
+}
+
+template <int L, int FAM, bool MIXED, int ALG>
+__global__ void __launch_bounds__(WARP_TPB, (warp_ext_min_ctas<L, FAM, MIXED, ALG>())) k_solve_warp_ext(SolveArgs a)
 {
     warp_lanes<typename warp_ext_solver<L, FAM, MIXED, ALG>::type, L, MIXED>(a);
 }
