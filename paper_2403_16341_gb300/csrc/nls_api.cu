@@ -21,6 +21,7 @@
 
 #include "../../include/nls.h"
 #include "nls_internal.h"
+#include "nls_ring.h"
 
 // (no `using namespace nls`: its exp overloads must not leak into global lookup)
 using nls::KernelInfo;
@@ -104,10 +105,8 @@ struct nls_batch {
     unsigned long long *d_ctr = nullptr; // [RING]
     unsigned long long *h_ctr = nullptr; // pinned mirror
     std::vector<int64_t> owner;          // ring slot -> request id (0 = free)
-    int ring_pos = 0;
-    int ring_zeroed = 0;                 // entries [ring_pos, ring_zeroed) are free and zero,
-    cudaStream_t zero_on = nullptr;      // by a memset on this stream,
-    cudaEvent_t zero_ev = nullptr;       // which launches on others wait for
+    nls::CounterRing<cudaStream_t> ring{RING, RING_BLOCK};
+    cudaEvent_t zero_ev = nullptr;       // follows the ring's last memset
     // nls_solve_host / nls_solve_host_async: staging blocks not in use (by
     // size), events not in use, and the requests in flight
     std::multimap<size_t, void *> stage_free;
@@ -276,24 +275,18 @@ static int wait_event(nls_batch *h, cudaEvent_t ev, int timeout_ms)
     }
 }
 
-// Reserve `count` consecutive ring entries, zero in the launch stream's order.
-// Blocks of the ring are zeroed on the launch stream as the position reaches
-// them (once per RING_BLOCK entries, so a flush needs no memset of its own);
-// requests still owning entries of such a block are waited for and their
-// solved counts kept on the host first.  What a stream capture records zeroes
-// its own entries, so a block is only taken up to them.
+// Reserve `count` consecutive ring entries, zero in the launch stream's order
+// (nls_ring.h); requests still owning entries that are to be zeroed are waited
+// for and their solved counts kept on the host first.
 static int ring_take(nls_batch *h, int count, bool captured, int *start)
 {
     if (count > RING) return fail(h, NLS_E_INVALID, "too many requests in one flush (%d)", count / 2);
-    if (h->ring_pos + count > RING) h->ring_pos = h->ring_zeroed = 0;
-    const int s = h->ring_pos;
-    const cudaStream_t st = launch_stream(h);
-    if (s + count > h->ring_zeroed) {
-        const int z0 = h->ring_zeroed;
-        const int z1 = captured ? s + count : std::min(RING, (s + count + RING_BLOCK - 1) / RING_BLOCK * RING_BLOCK);
-        for (int i = z0; i < z1; ++i) {
+    struct Ops {
+        nls_batch *h;
+        int release(int i)
+        {
             const int64_t id = h->owner[i];
-            if (!id) continue;
+            if (!id) return NLS_OK;
             auto it = h->reqs.find(id);
             if (it != h->reqs.end() && it->second.slot >= 0) {
                 Request &r = it->second;
@@ -303,19 +296,22 @@ static int ring_take(nls_batch *h, int count, bool captured, int *start)
                 r.slot = -1;
             }
             h->owner[i] = 0;
+            return NLS_OK;
         }
-        if (!captured) {
+        int zero(int first, int end, cudaStream_t st)
+        {
             if (!h->zero_ev) NLS_CUDA(h, cudaEventCreateWithFlags(&h->zero_ev, cudaEventDisableTiming));
-            NLS_CUDA(h, cudaMemsetAsync(h->d_ctr + z0, 0, sizeof(unsigned long long) * (z1 - z0), st));
+            NLS_CUDA(h, cudaMemsetAsync(h->d_ctr + first, 0, sizeof(unsigned long long) * (end - first), st));
             NLS_CUDA(h, cudaEventRecord(h->zero_ev, st));
-            h->zero_on = st;
+            return NLS_OK;
         }
-        h->ring_zeroed = z1;
-    }
-    if (!captured && st != h->zero_on) NLS_CUDA(h, cudaStreamWaitEvent(st, h->zero_ev, 0));
-    h->ring_pos = s + count;
-    *start = s;
-    return NLS_OK;
+        int after_zero(cudaStream_t st)
+        {
+            NLS_CUDA(h, cudaStreamWaitEvent(st, h->zero_ev, 0));
+            return NLS_OK;
+        }
+    };
+    return h->ring.take(count, launch_stream(h), captured, Ops{h}, start);
 }
 
 // Refill threshold of a request's persistent thread-tiled grid: the caller's, if set.

@@ -1,0 +1,53 @@
+"""The ring of request counters on the GPU: flushes that take entries zeroed on
+another stream, reuse of entries that kernels wrote."""
+import numpy as np
+import pytest
+
+from paper_2403_16341_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+NEWTON = 0
+ENTRIES = 2  # of the ring, per request
+BLOCK = 1 << 12  # entries zeroed at a time
+
+
+@pytest.fixture()
+def solver():
+    import paper_2403_16341_gb300 as nls
+    s = nls.Solver(0)  # a ring of its own
+    yield s
+    s.close()
+
+
+def on_gpu(b):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(b.params)).cuda(), torch.from_numpy(np.ascontiguousarray(b.u0)).cuda()
+
+
+def test_rest_of_a_block_zeroed_on_the_second_solve_stream(solver):
+    # a host request of 2^18 instances in flight, its second chunk (on the second
+    # solve stream) the one that crosses into a block of the ring; then 2,100
+    # requests in one flush on the handle's stream
+    import torch
+
+    import paper_2403_16341_gb300 as nls
+    b = I.square_batch(2, 5)
+    p, u0 = on_gpu(b)
+    u = u0.clone()
+    for _ in range(BLOCK // ENTRIES - 1):
+        r = solver.submit(nls.NLS_SQUARE, p, u, NEWTON)
+        solver.flush()
+        solver.wait(r)
+    big = I.square_batch(2, 1 << 18)
+    hu = big.u0.copy()
+    hreq = nls.nls_solve_host_async(solver.h, big.family, big.params.ctypes.data, hu.ctypes.data, big.n, big.batch,
+                                    NEWTON, 1e-10, 50)
+    us = [u0.clone() for _ in range(2100)]
+    reqs = [solver.submit(nls.NLS_SQUARE, p, v, NEWTON) for v in us]
+    solver.flush()
+    assert [solver.wait(r) for r in reqs] == [b.batch] * len(us)
+    assert nls.nls_status(solver.h, hreq) == big.batch
+    want = np.sqrt(b.params)
+    assert np.abs(torch.stack(us).cpu().numpy() - want).max() < 1e-9
+    assert np.abs(hu - np.sqrt(big.params)).max() < 1e-9
