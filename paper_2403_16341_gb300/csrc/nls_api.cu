@@ -52,6 +52,7 @@ struct Request {
     int slot = -1;                         // first of 2 ring entries (solved, work counter)
     std::shared_ptr<cudaEvent_t> done;     // recorded after the request's group
     bool launched = false;
+    bool captured = false;                 // recorded by a stream capture: `done` cannot be waited for
     long long solved_final = -1;           // captured when the ring slot is reused
 };
 
@@ -290,8 +291,10 @@ static int ring_take(nls_batch *h, int count, bool captured, int *start)
             auto it = h->reqs.find(id);
             if (it != h->reqs.end() && it->second.slot >= 0) {
                 Request &r = it->second;
-                NLS_CUDA(h, cudaEventSynchronize(*r.done));
-                r.solved_final = (long long)h->h_ctr[r.slot];
+                if (!r.captured) {
+                    NLS_CUDA(h, cudaEventSynchronize(*r.done));
+                    r.solved_final = (long long)h->h_ctr[r.slot];
+                }
                 h->owner[r.slot] = h->owner[r.slot + 1] = 0;
                 r.slot = -1;
             }
@@ -622,6 +625,7 @@ static int flush_pending(nls_batch *h)
         r.args.solved = h->d_ctr + r.slot;
         r.done = ev;
         r.launched = true;
+        r.captured = captured;
         rs.push_back(&r);
     }
     std::vector<int> grids;
@@ -631,8 +635,9 @@ static int flush_pending(nls_batch *h)
         NLS_CUDA(h, cudaMemsetAsync(h->d_ctr + s0, 0, sizeof(unsigned long long) * 2 * nreq, launch_stream(h)));
     // A lone request is launched directly: one kernel and one copy cost less on
     // the host than building, updating and launching a graph of them (1,024
-    // cubic n = 3 systems by Newton, the whole call: 58.5 -> 52.6 us).
-    rc = h->opt.graph && nreq > 1 ? launch_graph(h, rs, grids, s0, 2 * nreq)
+    // cubic n = 3 systems by Newton, the whole call: 58.5 -> 52.6 us).  So is what
+    // a capture records: it becomes part of the caller's own graph.
+    rc = h->opt.graph && nreq > 1 && !captured ? launch_graph(h, rs, grids, s0, 2 * nreq)
                                   : launch_direct(h, rs, grids, s0, 2 * nreq, captured);
     if (rc) return rc;
     bool any_poly = false;

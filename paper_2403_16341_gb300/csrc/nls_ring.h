@@ -14,14 +14,18 @@ namespace nls {
 // stream zeroed, then a block that it zeroes itself.  The memset of the later
 // block is therefore ordered after the earlier one's, and one event, recorded
 // behind it, stands for both.
-// What a stream capture records zeroes its own entries, so a block is only taken
-// up to them.
+//
+// A flush recorded by a stream capture zeroes its own entries each time it
+// runs.  Its replays also write them at times that the ring does not see,
+// before and after they are handed out again: from the first such flush on,
+// every flush zeroes exactly its own entries.
 template <class Stream>
 struct CounterRing {
     int size, block;
     int pos = 0, zeroed = 0;
     bool any = false;      // a memset was made, on:
     Stream zero_on{};
+    bool recorded = false; // a capture has recorded a flush
 
     CounterRing(int size_, int block_) : size(size_), block(block_) {}
 
@@ -33,11 +37,13 @@ struct CounterRing {
     int take(int count, Stream st, bool captured, Ops &&ops, int *start)
     {
         if (pos + count > size) pos = zeroed = 0;
+        recorded = recorded || captured;
+        if (recorded) zeroed = pos;
         if (!captured && any && st != zero_on)
             if (int rc = ops.after_zero(st)) return rc;
         const int end = pos + count;
         if (end > zeroed) {
-            const int z1 = captured ? end : std::min(size, (end + block - 1) / block * block);
+            const int z1 = recorded ? end : std::min(size, (end + block - 1) / block * block);
             for (int i = zeroed; i < z1; ++i)
                 if (int rc = ops.release(i)) return rc;
             if (!captured) {

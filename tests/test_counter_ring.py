@@ -63,11 +63,12 @@ struct Model {
         join(known[st], event);
         return 0;
     }
-    // a flush on `st` uses the entries
-    void use(int first, int count, int st)
+    // a flush on `st` uses the entries (recorded by a capture: after a memset of its own)
+    void use(int first, int count, int st, bool recorded = false)
     {
         issue(st); // picks up what the host is ordered after
         for (int i = first; i < first + count; ++i) {
+            if (recorded) continue;
             if (!zero[i]) { std::printf("entry %d is handed out dirty\n", i); std::exit(1); }
             if (!after(st, zeroed_by[i])) { std::printf("entry %d: not ordered after its memset\n", i); std::exit(1); }
         }
@@ -105,6 +106,21 @@ int main(int argc, char **argv)
     } else if (kind == 1) { // one stream: one memset per block
         for (int i = 0; i < 3 * size / 2; ++i) flush(2, 0);
         std::printf("%d\n", m.memsets);
+    } else if (kind == 1000) { // one stream, with flushes that a capture recorded, replayed at any time
+        std::mt19937 rng(block);
+        std::vector<std::pair<int, int>> recorded;
+        for (int i = 0; i < 4000; ++i) {
+            const int count = 2 * (1 + rng() % 4);
+            if (i > 100 && recorded.size() < 3 && rng() % 8 == 0) {
+                if (ring.take(count, 0, true, Ops{&m}, &s)) std::exit(2);
+                recorded.push_back({s, count});
+            } else if (!recorded.empty() && rng() % 3 == 0) {
+                const auto r = recorded[rng() % recorded.size()];
+                m.use(r.first, r.second, 0, true);
+            } else {
+                flush(count, 0);
+            }
+        }
     } else { // any order of streams and sizes over many laps
         std::mt19937 rng(kind);
         for (int i = 0; i < 4000; ++i) {
@@ -148,3 +164,8 @@ def test_one_memset_per_block(harness):
 @pytest.mark.parametrize("size,block", [(64, 16), (256, 64), (1024, 64)])
 def test_any_order_of_streams(harness, seed, size, block):
     run(harness, seed, size, block)
+
+
+@pytest.mark.parametrize("block", [16, 64, 256])
+def test_replays_of_a_captured_flush(harness, block):
+    run(harness, 1000, 1024, block)

@@ -51,3 +51,67 @@ def test_rest_of_a_block_zeroed_on_the_second_solve_stream(solver):
     want = np.sqrt(b.params)
     assert np.abs(torch.stack(us).cpu().numpy() - want).max() < 1e-9
     assert np.abs(hu - np.sqrt(big.params)).max() < 1e-9
+
+
+@pytest.mark.parametrize("lone", [True, False])
+def test_captured_flush_replays_beside_direct_ones(lone):
+    # a flush recorded by a stream capture: each replay solves from the u at that
+    # time; direct flushes between replays, through a whole lap of the ring, are
+    # right as well
+    import torch
+
+    import paper_2403_16341_gb300 as nls
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        solver = nls.Solver(0)
+        solver.set_option(nls.NLS_OPT_CTAS_PER_SM, 1)
+        b = I.square_batch(2, 40000)  # several waves: a work counter
+        p, u0 = on_gpu(b)
+        groups = [u0.clone() for _ in range(1 if lone else 3)]
+        stat = torch.empty(b.batch, dtype=torch.int32, device="cuda")
+        small = I.square_batch(2, 5)
+        sp, su0 = on_gpu(small)
+        su = su0.clone()
+
+        def direct():
+            su.copy_(su0)
+            r = solver.submit(nls.NLS_SQUARE, sp, su, NEWTON)
+            solver.flush()
+            assert solver.wait(r) == small.batch
+
+        direct()
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            for v in groups:
+                solver.submit(nls.NLS_SQUARE, p, v, NEWTON, 1e-10, 50, (stat, None, None, None))
+            solver.flush()
+        want = np.sqrt(b.params)
+
+        def replay():
+            for v in groups:
+                v.copy_(u0)
+            stat.fill_(-1)
+            g.replay()
+            st.synchronize()
+            for v in groups:
+                assert np.abs(v.cpu().numpy() - want).max() < 1e-9
+            assert (stat == 0).all()
+
+        for _ in range(3):
+            replay()
+            direct()
+        big = u0.clone()
+        for i in range((1 << 16) // ENTRIES + 8):
+            if i % 4096 == 0:
+                replay()
+                big.copy_(u0)
+                r = solver.submit(nls.NLS_SQUARE, p, big, NEWTON)
+                solver.flush()
+                assert solver.wait(r) == b.batch
+                assert np.abs(big.cpu().numpy() - want).max() < 1e-9
+            else:
+                direct()
+        replay()
+        st.synchronize()
+        solver.close()
