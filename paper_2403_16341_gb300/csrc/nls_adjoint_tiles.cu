@@ -188,7 +188,8 @@ template <int R, int FAM>
 static cudaError_t launch_adjoint_cta_rf(const AdjointTileArgs &g, cudaStream_t st)
 {
     const int smem = cta_smem_bytes<false, R>();
-    static const cudaError_t attr = cudaFuncSetAttribute(
+    // more than 48 KB needs an opt-in, on the device that is current
+    const cudaError_t attr = cudaFuncSetAttribute(
         reinterpret_cast<const void *>(&k_adjoint_cta<R, FAM>), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (attr != cudaSuccess) return attr;
     int dev = 0, sms = 0, occ = 0;

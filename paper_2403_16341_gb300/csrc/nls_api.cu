@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "../../include/nls.h"
+#include "nls_attr.h"
 #include "nls_internal.h"
 #include "nls_ring.h"
 
@@ -116,6 +117,7 @@ struct nls_batch {
     // cached executable graphs by request-shape signature
     std::map<std::string, cudaGraphExec_t> graphs;
     std::map<std::pair<const void *, int>, int> occ_cache; // by kernel and shared memory
+    nls::SmemOptIns opt_ins;
     std::map<long long, Tuned> tuned;
     double *d_tune = nullptr; // autotuner scratch for a prefix of u
     size_t tune_bytes = 0;
@@ -243,6 +245,15 @@ static int select_kernel(nls_batch *h, int family, int n, int alg, KernelInfo *o
     return NLS_OK;
 }
 
+// Makes a kernel launchable on the handle's device, which is current.
+static int prepare_kernel(nls_batch *h, const KernelInfo &k)
+{
+    return h->opt_ins.ensure(k.func, k.smem_most, [h](const void *f, int bytes) {
+        NLS_CUDA(h, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+        return (int)NLS_OK;
+    });
+}
+
 static int occupancy(nls_batch *h, const KernelInfo &k, int *occ)
 {
     const auto key = std::make_pair(k.func, k.smem);
@@ -340,6 +351,8 @@ static int plan_grids(nls_batch *h, const std::vector<Request *> &rs, std::vecto
     for (size_t i = 0; i < rs.size(); ++i) {
         Request &r = *rs[i];
         if (r.args.batch == 0 || r.poly) continue; // a poly request runs its own chain
+        int rc = prepare_kernel(h, r.kern);
+        if (rc) return rc;
         const int64_t ctas = (r.args.batch + r.kern.per_cta - 1) / r.kern.per_cta;
         const bool persistent = h->opt.persistent && live == 1 && r.refill != REFILL_STATIC;
         if (!persistent) {
@@ -349,7 +362,7 @@ static int plan_grids(nls_batch *h, const std::vector<Request *> &rs, std::vecto
             continue;
         }
         int occ = 0;
-        int rc = occupancy(h, r.kern, &occ);
+        rc = occupancy(h, r.kern, &occ);
         if (rc) return rc;
         if (h->opt.ctas_per_sm > 0) occ = std::min(occ, h->opt.ctas_per_sm);
         grids[i] = (int)std::min<int64_t>(ctas, (int64_t)std::max(occ, 1) * h->sms);
@@ -540,6 +553,8 @@ static int launch_poly(nls_batch *h, Request &r)
     // first stage on the whole batch
     KernelInfo k0 = stage_kernel(stages[0]);
     if (!k0.launch) return fail(h, NLS_E_UNSUPPORTED, "no poly stage kernel for family %d, n = %d", r.family, n);
+    int rc = prepare_kernel(h, k0);
+    if (rc) return rc;
     a.alg = stages[0];
     a.counter = nullptr;
     a.refill_below = 0;
@@ -551,7 +566,8 @@ static int launch_poly(nls_batch *h, Request &r)
         const KernelInfo ks = stage_kernel(stages[sidx]);
         if (!ks.launch) return fail(h, NLS_E_UNSUPPORTED, "no poly stage kernel for family %d, n = %d", r.family, n);
         int occ = 0;
-        int rc = occupancy(h, ks, &occ);
+        rc = prepare_kernel(h, ks);
+        if (!rc) rc = occupancy(h, ks, &occ);
         if (rc) return rc;
         const int64_t ctas = (B + ks.per_cta - 1) / ks.per_cta;
         const int grid = (int)std::min<int64_t>(ctas, (int64_t)std::max(occ, 1) * h->sms);
@@ -715,7 +731,8 @@ static int tune_trial(nls_batch *h, const SolveArgs &base, int base_family, cons
     a.nfev = nullptr;
     a.ngrad = nullptr;
     int occ = 0;
-    int rc = occupancy(h, k, &occ);
+    int rc = prepare_kernel(h, k);
+    if (!rc) rc = occupancy(h, k, &occ);
     if (rc) return rc;
     const int64_t ctas = (S + k.per_cta - 1) / k.per_cta;
     const int grid = refill == REFILL_STATIC ? (int)std::min<int64_t>(ctas, INT32_MAX)

@@ -21,16 +21,12 @@ static KernelInfo cols_info(int n)
 {
     if (n < 1 || n > COL_NMAX) return KernelInfo{};
     constexpr int C = col_panel<MIXED>();
-    const void *f = reinterpret_cast<const void *>(&k_solve_cols<C, FAM, MIXED>);
-    // more than 48 KB of dynamic shared memory needs an opt-in, once per kernel
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, col_smem_bytes<C, MIXED>(COL_NMAX));
-    (void)attr;
     KernelInfo k;
     k.launch = &launch_cols<FAM, MIXED>;
-    k.func = f;
+    k.func = reinterpret_cast<const void *>(&k_solve_cols<C, FAM, MIXED>);
     k.block = 32 * col_warps<MIXED>(n);
     k.smem = col_smem_bytes<C, MIXED>(n);
+    k.smem_most = col_smem_bytes<C, MIXED>(COL_NMAX);
     k.per_cta = 1;
     return k;
 }

@@ -326,16 +326,11 @@ cudaError_t launch_cta_ext(const SolveArgs &a, int grid, cudaStream_t st)
 template <int R, int FAM, bool MIXED, int ALG>
 KernelInfo cta_ext_info()
 {
-    // more than 48 KB of dynamic shared memory needs an opt-in, once per kernel
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        reinterpret_cast<const void *>(&k_solve_cta_ext<R, FAM, MIXED, ALG>),
-        cudaFuncAttributeMaxDynamicSharedMemorySize, cta_smem_bytes<MIXED, R>());
-    (void)attr;
     KernelInfo k;
     k.launch = &launch_cta_ext<R, FAM, MIXED, ALG>;
     k.func = reinterpret_cast<const void *>(&k_solve_cta_ext<R, FAM, MIXED, ALG>);
     k.block = CTA_TPB;
-    k.smem = cta_smem_bytes<MIXED, R>();
+    k.smem = k.smem_most = cta_smem_bytes<MIXED, R>();
     k.per_cta = 1;
     return k;
 }
