@@ -55,10 +55,26 @@ constexpr int COL_NMAX = 128;
 template <bool MIXED>
 constexpr int col_chunk() { return MIXED ? 32 : 16; }
 
-// The multipliers' reciprocal pivot: in FP32 the hardware approximation
-// (pivot_rcp: its error is inside the FP32 LU's own rounding; a zero or
-// non-finite pivot is caught before it is used), in FP64 the rounded one.
-NLS_DI double pivot_rcp(double x) { return rcp(x); }
+// The multipliers' reciprocal pivot and whether the pivot is neither zero, an
+// infinity nor a NaN.  FP32: the hardware approximation (pivot_rcp: its error is
+// inside the FP32 LU's own rounding) where it and its result are normal numbers,
+// which it would flush otherwise (a pivot above 2^126 would zero its multipliers);
+// the rounded reciprocal elsewhere.  FP64: the rounded one.
+NLS_DI float pivot_reciprocal(float x, bool &ok)
+{
+    const uint32_t m = mag_bits(x);
+    if (m - 0x00800000u >= 0x7e800000u - 0x00800000u) { // not in [2^-126, 2^126)
+        if (m == 0u || m >= INF32_BITS) ok = false;
+        return rcp(x);
+    }
+    return pivot_rcp(x);
+}
+NLS_DI double pivot_reciprocal(double x, bool &ok)
+{
+    const uint64_t m = mag_bits(x);
+    if (m == 0u || m >= INF64_BITS) ok = false;
+    return rcp(x);
+}
 
 // Columns per panel.  A wider panel means fewer passes over the trailing
 // columns but a longer serial part (its own columns' update and factors).
@@ -480,7 +496,6 @@ struct ColSolver {
     NLS_DI void factor_panel(int k0, int kc, int p, SM &sm) const
     {
         const unsigned FULL = 0xffffffffu;
-        const K inf = inf_bits(P(0));
         const int par = p & 1;
         P v[C][SK];
         int pos[SK];
@@ -498,9 +513,7 @@ struct ColSolver {
                 int src, pslot, ppos;
                 find_pivot<SK>(v[0], pos, kk, src, pslot, ppos);
                 const P pv = __shfl_sync(FULL, pick<SK>(v[0], pslot), src);
-                const K pm = mag_bits(pv);
-                if (pm == K(0) || pm >= inf) ok = false;
-                const P r = pivot_rcp(pv);
+                const P r = pivot_reciprocal(pv, ok);
                 take_pivot<SK>(pos, kk, src, pslot, ppos);
                 // column kk is finished: multipliers of the rows that remain, U of
                 // the others, kept by row until the panel's end
@@ -557,9 +570,7 @@ struct ColSolver {
                 int src, pslot, ppos;
                 find_pivot<SK>(v[c], pos, kk, src, pslot, ppos);
                 const P pv = __shfl_sync(FULL, pick<SK>(v[c], pslot), src);
-                const K pm = mag_bits(pv);
-                if (pm == K(0) || pm >= inf) ok = false;
-                const P r = pivot_rcp(pv);
+                const P r = pivot_reciprocal(pv, ok);
                 take_pivot<SK>(pos, kk, src, pslot, ppos);
 #pragma unroll
                 for (int s = 0; s < SK; ++s)
