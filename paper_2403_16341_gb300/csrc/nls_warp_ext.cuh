@@ -29,8 +29,9 @@ namespace nls {
 // on return lane r's row holds its multipliers in the columns before its
 // final position `pos` and U from `pos` on; rc = 1 / pivot of row `pos`.
 // Same pivot choice as WarpSolver::lu_solve.  Returns false (segment-
-// uniform) on a zero or non-finite pivot.
-template <int L, class P, class SM>
+// uniform) on a zero or non-finite pivot.  FP64_RCP: the FP64 reciprocal on the
+// FP64 pipe; the bits are rcp's.
+template <int L, bool FP64_RCP = false, class P = double, class SM = void>
 NLS_DI bool warp_lu_factor(P (&a)[L], int r, int n, SM &sm, int &pos, P &rc)
 {
     using K = decltype(mag_bits(P(0)));
@@ -65,7 +66,9 @@ NLS_DI bool warp_lu_factor(P (&a)[L], int r, int n, SM &sm, int &pos, P &rc)
                 for (int c = k; c < L; ++c) sm.prow[c] = a[c];
             }
             __syncwarp();
-            const P pr = rcp(sm.prow[k]);
+            P pr;
+            if constexpr (FP64_RCP && sizeof(P) == 8) pr = __drcp_rn(sm.prow[k]);
+            else pr = rcp(sm.prow[k]);
             if (cand && pos == k && !is_piv) pos = ppos;
             if (is_piv) {
                 pos = k;
@@ -272,7 +275,12 @@ struct WarpSolverBroyden : WarpSolverExtBase<L, FAM, MIXED> {
                 this->jacobian_row(a, sm);
                 int pos;
                 P rc;
-                const bool ok = warp_lu_factor<L>(a, r, n, sm, pos, rc);
+                // once per solve, between the passes' products: the integer
+                // reciprocal, which frees the FP64 pipe in a loop of factorisations,
+                // costs more here than it frees (20,000 FP64 systems, modified
+                // Broyden: Bratu n = 32 6.28 ms against 6.00, cubic n = 32 8.87
+                // against 8.49, Bratu n = 24 4.55 against 4.33)
+                const bool ok = warp_lu_factor<L, true>(a, r, n, sm, pos, rc);
                 // column j of J^-1 lands in lane r's own row r of the transpose
                 // buffer (a runtime loop: the solve is emitted once)
 #pragma unroll 1
