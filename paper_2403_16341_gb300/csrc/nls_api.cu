@@ -445,16 +445,27 @@ static int launch_graph(nls_batch *h, const std::vector<Request *> &rs, const st
     return NLS_OK;
 }
 
-constexpr int MIRROR_MAX_GRID = 4096;
+// Whether a lone request counts its solved instances in the pinned mirror
+// itself, one add per warp (CTA tiling: per instance) over the link, instead of
+// in device memory with a 16-byte copy behind the kernel.  The copy costs about
+// 3 us, so do some 512 adds that arrive together, as those of a warp-tiled batch
+// of similar instances do (square n = 16, mixed, the whole call, adds against
+// copy: 512 instances 70.9 / 73.6 us, 1,024 74.1 / 74.2, 2,048 80.6 / 75.9,
+// 4,096 97.0 / 86.5).  A thread-tiled warp adds 32 instances at once and the
+// warps end apart: equal at 1,024 and 4,096 adds (cubic n = 3, 32,768: 55.0 / 54.8,
+// 131,072: 98.4 / 98.5), ahead where a refill spreads the ends (square n = 8).
+static bool counts_in_mirror(const Request &r, int grid)
+{
+    if (r.tiles == NLS_TILE_THREAD) return grid <= 4096; // CTAs of one warp
+    if (r.tiles == NLS_TILE_WARP) return (int64_t)grid * r.kern.block / 32 <= 512;
+    return r.args.batch <= 512;
+}
 
 static int launch_direct(nls_batch *h, const std::vector<Request *> &rs, const std::vector<int> &grids, int s0,
                          int nctr, bool captured)
 {
     const cudaStream_t st = launch_stream(h);
-    // A lone request on a small grid counts its solved instances in the pinned
-    // mirror itself: one add per warp (CTA tiling: per instance) over the link
-    // instead of a copy behind the kernel.
-    const bool mirror = !captured && rs.size() == 1 && grids[0] > 0 && grids[0] <= MIRROR_MAX_GRID;
+    const bool mirror = !captured && rs.size() == 1 && grids[0] > 0 && counts_in_mirror(*rs[0], grids[0]);
     if (mirror) {
         h->h_ctr[rs[0]->slot] = 0;
         rs[0]->args.solved = h->h_ctr + rs[0]->slot;
