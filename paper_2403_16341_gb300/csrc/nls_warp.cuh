@@ -34,7 +34,13 @@
 
 namespace nls {
 
-constexpr int WARP_TPB = 64; // 2 warps per CTA: they never wait on each other
+// Threads per CTA; its warps never wait on each other.  Two warps, so that a
+// batch of about a wave spreads evenly (1,000 FP64 n = 32 systems: 309 us, 350
+// with four); four with 16 FP64 lanes, whose instances are short: a flush of many
+// small requests launches half the CTAs (8,192 FP64 systems of n = 2..16,
+// Newton / backtracking: 479 / 485 -> 446 / 447 us, n = 2..12: 382 -> 363).
+template <int L, bool MIXED>
+constexpr int warp_tpb() { return L == 16 && !MIXED ? 128 : 64; }
 
 // One segment's shared memory.  U holds the pivot row of every step k, from
 // its column k on (the factor U by positions), at slot VEC - 1 + (column - k),
@@ -650,7 +656,7 @@ struct WarpSolver {
 template <int L, bool MIXED, int FAM>
 constexpr int warp_smem_bytes()
 {
-    constexpr int bytes = (WARP_TPB / 32) * (32 / L) * (int)sizeof(WarpSmem<L, MIXED, FAM>);
+    constexpr int bytes = (warp_tpb<L, MIXED>() / 32) * (32 / L) * (int)sizeof(WarpSmem<L, MIXED, FAM>);
     static_assert(bytes <= 48 * 1024, "no opt-in beyond 48 KB is made for these kernels");
     return bytes;
 }
@@ -679,7 +685,7 @@ NLS_DI void warp_lanes(SolveArgs &a)
     bool have = false, exhausted = false, first = true;
     int64_t k = -1;
     unsigned long long local_solved = 0;
-    const int64_t warp_global = (int64_t)blockIdx.x * (WARP_TPB / 32) + warp;
+    const int64_t warp_global = (int64_t)blockIdx.x * (warp_tpb<L, MIXED>() / 32) + warp;
 
     for (;;) {
         // segments are the units of work: one ballot bit per segment leader
@@ -743,14 +749,23 @@ NLS_DI void warp_lanes(SolveArgs &a)
 
 // CTAs per SM that the compiler makes room for (0: its own choice).  The
 // 32-lane FP64 kernels take the 6 that the cubic's shared memory allows (164
-// registers instead of 222, which held 4).  Mixed, 8 CTAs (128 registers and a
-// spill) measured 2% faster on n = 32 alone but 5% slower in a flush of many
-// sizes.
-template <int L, bool MIXED>
-constexpr int warp_min_ctas() { return L == 32 && !MIXED ? 6 : 0; }
+// registers instead of 222, which held 4: 5,000 n = 27 systems 916 us against
+// 1,151).  Mixed, 8 CTAs (128 registers and a spill) measured 2% faster on n = 32
+// alone but 5% slower in a flush of many sizes.  16 lanes: sixteen FP64 warps per
+// SM (120 registers; left alone, Bratu's kernel took 154, which held twelve), and
+// 24 mixed ones of the families without a matrix of their own (80 registers
+// instead of 89 to 96; 20,000 systems of n = 16: square 196 -> 184 us, Bratu 175 ->
+// 171).
+template <int L, int FAM, bool MIXED>
+constexpr int warp_min_ctas()
+{
+    if (L == 32) return MIXED ? 0 : 6;
+    if (L == 16) return !MIXED ? 4 : FAM == FAM_CUBIC ? 0 : 12;
+    return 0;
+}
 
 template <int L, int FAM, bool MIXED>
-__global__ void __launch_bounds__(WARP_TPB, warp_min_ctas<L, MIXED>()) k_solve_warp(SolveArgs a)
+__global__ void __launch_bounds__((warp_tpb<L, MIXED>()), (warp_min_ctas<L, FAM, MIXED>())) k_solve_warp(SolveArgs a)
 {
     warp_lanes<WarpSolver<L, FAM, MIXED>, L, MIXED>(a);
 }

@@ -7,7 +7,7 @@ namespace nls {
 template <int L, int FAM>
 static cudaError_t launch_warp_fp64(const SolveArgs &a, int grid, cudaStream_t st)
 {
-    k_solve_warp<L, FAM, false><<<grid, WARP_TPB, warp_smem_bytes<L, false, FAM>(), st>>>(a);
+    k_solve_warp<L, FAM, false><<<grid, warp_tpb<L, false>(), warp_smem_bytes<L, false, FAM>(), st>>>(a);
     return cudaGetLastError();
 }
 
@@ -17,9 +17,9 @@ static KernelInfo info_fp64()
     KernelInfo k;
     k.launch = &launch_warp_fp64<L, FAM>;
     k.func = reinterpret_cast<const void *>(&k_solve_warp<L, FAM, false>);
-    k.block = WARP_TPB;
+    k.block = warp_tpb<L, false>();
     k.smem = warp_smem_bytes<L, false, FAM>();
-    k.per_cta = (WARP_TPB / 32) * (32 / L);
+    k.per_cta = (warp_tpb<L, false>() / 32) * (32 / L);
     return k;
 }
 
