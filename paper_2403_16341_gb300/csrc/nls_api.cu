@@ -117,7 +117,7 @@ struct nls_batch {
     // cached executable graphs by request-shape signature
     std::map<std::string, cudaGraphExec_t> graphs;
     std::map<std::pair<const void *, int>, int> occ_cache; // by kernel and shared memory
-    nls::SmemOptIns opt_ins;
+    nls::SmemOptIns opt_ins, splits;
     std::map<long long, Tuned> tuned;
     double *d_tune = nullptr; // autotuner scratch for a prefix of u
     size_t tune_bytes = 0;
@@ -248,8 +248,13 @@ static int select_kernel(nls_batch *h, int family, int n, int alg, KernelInfo *o
 // Makes a kernel launchable on the handle's device, which is current.
 static int prepare_kernel(nls_batch *h, const KernelInfo &k)
 {
-    return h->opt_ins.ensure(k.func, k.smem_most, [h](const void *f, int bytes) {
+    int rc = h->opt_ins.ensure(k.func, k.smem_most, [h](const void *f, int bytes) {
         NLS_CUDA(h, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+        return (int)NLS_OK;
+    });
+    if (rc) return rc;
+    return h->splits.ensure_if(k.widest_smem, k.func, [h](const void *f) {
+        NLS_CUDA(h, cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
         return (int)NLS_OK;
     });
 }

@@ -1,6 +1,7 @@
 // nls_attr.h -- function attributes that a kernel needs before its launch.
 #pragma once
 
+#include <climits>
 #include <set>
 
 namespace nls {
@@ -20,6 +21,12 @@ struct SmemOptIns {
         const int rc = set(func, bytes);
         if (!rc) done.insert(func);
         return rc;
+    }
+    // Likewise for another attribute, set(func), of the kernels that want it.
+    template <class Set>
+    int ensure_if(bool wanted, const void *func, Set &&set)
+    {
+        return ensure(func, wanted ? INT_MAX : 0, [&](const void *f, int) { return set(f); });
     }
 };
 

@@ -15,6 +15,7 @@ struct KernelInfo {
     int block = 0;     // threads per CTA
     int smem = 0;      // dynamic shared memory bytes
     int smem_most = 0; // most dynamic shared memory of any launch of func, where that is above 48 KB for some n
+    bool widest_smem = false; // an SM running it is configured for the most shared memory
     int per_cta = 0;   // instances per CTA per round (static grids)
 };
 

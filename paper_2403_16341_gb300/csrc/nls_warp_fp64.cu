@@ -19,6 +19,13 @@ static KernelInfo info_fp64()
     k.func = reinterpret_cast<const void *>(&k_solve_warp<L, FAM, false>);
     k.block = warp_tpb<L, false>();
     k.smem = warp_smem_bytes<L, false, FAM>();
+    // An SM's split between L1 and shared memory changes only when the SM is idle,
+    // and the driver takes the smallest split that a kernel's occupancy needs.
+    // Beside a 32-lane kernel of another family, which needs half of what the cubic
+    // does, the cubic's CTAs then waited for it to drain (one flush, Bratu n = 32,
+    // 664 systems, then cubic n = 32, 279: 627 us, 321 in the other order).  With
+    // one split for all 32-lane kernels: 321 us in both.
+    k.widest_smem = L == 32;
     k.per_cta = (warp_tpb<L, false>() / 32) * (32 / L);
     return k;
 }
