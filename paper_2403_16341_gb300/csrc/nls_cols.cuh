@@ -55,27 +55,6 @@ constexpr int COL_NMAX = 128;
 template <bool MIXED>
 constexpr int col_chunk() { return MIXED ? 32 : 16; }
 
-// The multipliers' reciprocal pivot and whether the pivot is neither zero, an
-// infinity nor a NaN.  FP32: the hardware approximation (pivot_rcp: its error is
-// inside the FP32 LU's own rounding) where it and its result are normal numbers,
-// which it would flush otherwise (a pivot above 2^126 would zero its multipliers);
-// the rounded reciprocal elsewhere.  FP64: the rounded one.
-NLS_DI float pivot_reciprocal(float x, bool &ok)
-{
-    const uint32_t m = mag_bits(x);
-    if (m - 0x00800000u >= 0x7e800000u - 0x00800000u) { // not in [2^-126, 2^126)
-        if (m == 0u || m >= INF32_BITS) ok = false;
-        return rcp(x);
-    }
-    return pivot_rcp(x);
-}
-NLS_DI double pivot_reciprocal(double x, bool &ok)
-{
-    const uint64_t m = mag_bits(x);
-    if (m == 0u || m >= INF64_BITS) ok = false;
-    return rcp(x);
-}
-
 // Columns per panel.  A wider panel means fewer passes over the trailing
 // columns but a longer serial part (its own columns' update and factors).
 // Measured on 16,384 Bratu systems of n = 64..128: mixed 13.9 / 12.8 / 18 ms
