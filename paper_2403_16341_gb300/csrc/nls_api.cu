@@ -184,10 +184,20 @@ static int dev_alloc(nls_batch *h, void **p, size_t bytes)
     return NLS_OK;
 }
 
+// The CTA-tiled Newton-family kernel for a flush (or a tuning trial) of `instances`
+// such instances.
+static KernelInfo cta_choice(const nls_batch *h, int family, int n, int alg, int64_t instances)
+{
+    const bool mixed = (alg & NLS_MIXED) != 0;
+    if (mixed && instances <= nls::panel_most(family, n, (alg & NLS_REFINE) != 0, h->sms))
+        return nls::panel_kernel(family, n);
+    return cta_kernel(family, n, mixed);
+}
+
 // Pick the kernel for one request: a forced tiling flag, else the autotuned
 // choice for (family, n, algorithm, precision), else thread (n <= 8), warp
 // (n <= 32) or CTA (n <= 128).
-static int select_kernel(nls_batch *h, int family, int n, int alg, KernelInfo *out, int *tiles_out,
+static int select_kernel(nls_batch *h, int family, int n, int64_t batch, int alg, KernelInfo *out, int *tiles_out,
                          int *lanes_out, int *refill_out, double *rate_out)
 {
     const bool mixed = (alg & NLS_MIXED) != 0;
@@ -235,7 +245,7 @@ static int select_kernel(nls_batch *h, int family, int n, int alg, KernelInfo *o
         if (n > 32) return fail(h, NLS_E_UNSUPPORTED, "warp tiling holds n <= 32 (n = %d)", n);
         *out = warp_kernel(family, n, mixed, lanes);
     } else {
-        *out = cta_kernel(family, n, mixed);
+        *out = cta_choice(h, family, n, alg, batch);
     }
     if (!out->launch) return fail(h, NLS_E_UNSUPPORTED, "no kernel for family %d, n = %d", family, n);
     if (tiles_out) *tiles_out = tiles;
@@ -350,12 +360,20 @@ static int default_refill(const nls_batch *h, int family, int alg)
 static int plan_grids(nls_batch *h, const std::vector<Request *> &rs, std::vector<int> &grids)
 {
     int live = 0;
+    int64_t cta_instances = 0; // mixed precision, Newton family
+    auto panel_or_columns = [](const Request &r) {
+        return r.tiles == NLS_TILE_CTA && (r.alg_flags & NLS_MIXED) && r.args.alg < NLS_POTRA_PTAK;
+    };
     for (Request *r : rs)
-        if (r->args.batch > 0 && !r->poly) ++live;
+        if (r->args.batch > 0 && !r->poly) {
+            ++live;
+            if (panel_or_columns(*r)) cta_instances += r->args.batch;
+        }
     grids.assign(rs.size(), 0);
     for (size_t i = 0; i < rs.size(); ++i) {
         Request &r = *rs[i];
         if (r.args.batch == 0 || r.poly) continue; // a poly request runs its own chain
+        if (panel_or_columns(r)) r.kern = cta_choice(h, r.family, r.args.n, r.alg_flags, cta_instances);
         int rc = prepare_kernel(h, r.kern);
         if (rc) return rc;
         const int64_t ctas = (r.args.batch + r.kern.per_cta - 1) / r.kern.per_cta;
@@ -814,7 +832,7 @@ static int enqueue(nls_batch *h, int family, const double *params, double *u, in
 {
     int rc = 0;
     Request r;
-    rc = select_kernel(h, family, n, alg, &r.kern, &r.tiles, &r.lanes, &r.refill, &r.rate);
+    rc = select_kernel(h, family, n, batch, alg, &r.kern, &r.tiles, &r.lanes, &r.refill, &r.rate);
     if (rc) return rc;
     r.family = family;
     r.id = h->next_id++;
@@ -1198,7 +1216,7 @@ int nls_autotune(nls_handle h, int family, const double *params, double *u, int 
                                               : nls::cta_ext_kernel(family, n, a, mixed);
         return c.tiles == NLS_TILE_THREAD ? thread_kernel(family, n, mixed, analytic)
                : c.tiles == NLS_TILE_WARP ? warp_kernel(family, n, mixed, c.lanes)
-                                          : cta_kernel(family, n, mixed);
+                                          : cta_choice(h, family, n, alg, S);
     };
     Tuned best;
     for (Tuned &c : cands) {

@@ -50,6 +50,28 @@ namespace nls {
 // One instance per CTA, n <= 128: the matrix by columns in shared memory
 // (nls_cols.cuh); block and shared memory depend on n.
 KernelInfo cta_kernel(int family, int n, bool mixed);
+// ... or, in mixed precision and n <= 96, in registers (nls_panel.cuh).
+KernelInfo panel_kernel(int family, int n);
+
+// The most mixed-precision instances, over all CTA-tiled requests of a flush, that
+// run on panel_kernel.  It has the lower latency, cta_kernel the throughput, so the
+// line is one wave of its CTAs (4 per SM up to n = 64, 2 up to n = 96; above that
+// the two are within 5%).  Trust region, time here / time of cta_kernel at a wave's
+// end and beyond: Bratu n = 64 608: 0.80, 1,000: 1.20; n = 48 0.89, 1.30; n = 96 304:
+// 0.91, 456: 1.37; cubic n = 96 0.76, 1.23.  The cubic up to n = 64 re-reads A with
+// more threads per instance here, and stays ahead for more waves: n = 33 1,000: 0.91,
+// 2,000: 1.07; n = 48 2,000: 0.95, 4,000: 1.03; n = 64 2,000: 0.93, 4,000: 0.99;
+// refined n = 48 and 64 1,000: 0.90 and 0.86, 2,000: 1.05 and 1.00; n = 32 2,000: 0.93,
+// n = 24 608: 0.69, 1,000: 1.12.  The smallest systems (refined, or asked for) are one
+// panel there and gain nothing: 50 systems of n = 8 0.91 (cubic) and 1.03 (Bratu),
+// n = 16 0.73 and 0.86.
+inline int64_t panel_most(int family, int n, bool refine, int sms)
+{
+    const bool cubic = family == FAM_CUBIC;
+    if (n > 96 || n < (cubic ? 8 : 9)) return 0;
+    const int waves = !cubic || n < 32 || n > 64 ? 1 : refine || n <= 40 ? 2 : 4;
+    return (int64_t)waves * (n <= 64 ? 4 : 2) * sms;
+}
 } // namespace nls
 
 namespace nls {

@@ -102,6 +102,22 @@ KernelInfo cta_kernel(int family, int n, bool mixed)
     }
 }
 
+KernelInfo panel_kernel_mixed_cubic(int n);
+KernelInfo panel_kernel_mixed_bratu(int n);
+KernelInfo panel_kernel_mixed_square(int n);
+KernelInfo panel_kernel_mixed_rosenbrock(int n);
+
+KernelInfo panel_kernel(int family, int n)
+{
+    switch (family) {
+    case FAM_CUBIC: return panel_kernel_mixed_cubic(n);
+    case FAM_BRATU: return panel_kernel_mixed_bratu(n);
+    case FAM_SQUARE: return panel_kernel_mixed_square(n);
+    case FAM_ROSENBROCK: return panel_kernel_mixed_rosenbrock(n);
+    default: return KernelInfo{};
+    }
+}
+
 KernelInfo warp_kernel(int family, int n, bool mixed, int lanes)
 {
     int L = lanes ? lanes : (n <= 8 ? 8 : n <= 16 ? 16 : 32);
