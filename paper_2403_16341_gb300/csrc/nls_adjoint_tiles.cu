@@ -40,7 +40,7 @@ struct AdjointTileArgs {
 // no residual is formed and A is not kept, so a segment needs the LU's rows in
 // shared memory only and ten CTAs share an SM.
 template <int L, int FAM>
-__global__ void __launch_bounds__((warp_tpb<L, false>())) k_adjoint_warp(AdjointTileArgs g)
+__global__ void __launch_bounds__((warp_tpb<L, FAM_SQUARE, false>())) k_adjoint_warp(AdjointTileArgs g)
 {
     using S = WarpSolver<L, FAM, false>;
     using SM = WarpSmem<L, false, FAM_SQUARE>; // without A
@@ -50,7 +50,7 @@ __global__ void __launch_bounds__((warp_tpb<L, false>())) k_adjoint_warp(Adjoint
     const int seg = lane / L;
     SM &sm = reinterpret_cast<SM *>(smem_raw)[warp * SEGS + seg];
     const unsigned FULL = 0xffffffffu;
-    const int64_t mine = ((int64_t)blockIdx.x * (warp_tpb<L, false>() / 32) + warp) * SEGS + seg;
+    const int64_t mine = ((int64_t)blockIdx.x * (warp_tpb<L, FAM_SQUARE, false>() / 32) + warp) * SEGS + seg;
     const bool real = mine < g.batch;
     const int64_t k = real ? mine : g.batch - 1;
     const int64_t B = g.batch;
@@ -109,9 +109,9 @@ __global__ void __launch_bounds__((warp_tpb<L, false>())) k_adjoint_warp(Adjoint
 template <int L, int FAM>
 static cudaError_t launch_adjoint_warp_lf(const AdjointTileArgs &g, cudaStream_t st)
 {
-    constexpr int per_cta = (warp_tpb<L, false>() / 32) * (32 / L);
+    constexpr int per_cta = (warp_tpb<L, FAM_SQUARE, false>() / 32) * (32 / L);
     const int64_t grid = (g.batch + per_cta - 1) / per_cta;
-    k_adjoint_warp<L, FAM><<<(unsigned)grid, warp_tpb<L, false>(), warp_smem_bytes<L, false, FAM_SQUARE>(), st>>>(g);
+    k_adjoint_warp<L, FAM><<<(unsigned)grid, (warp_tpb<L, FAM_SQUARE, false>()), warp_smem_bytes<L, false, FAM_SQUARE>(), st>>>(g);
     return cudaGetLastError();
 }
 

@@ -37,10 +37,12 @@ namespace nls {
 // Threads per CTA; its warps never wait on each other.  Two warps, so that a
 // batch of about a wave spreads evenly (1,000 FP64 n = 32 systems: 309 us, 350
 // with four); four with 16 FP64 lanes, whose instances are short: a flush of many
-// small requests launches half the CTAs (8,192 FP64 systems of n = 2..16,
-// Newton / backtracking: 479 / 485 -> 446 / 447 us, n = 2..12: 382 -> 363).
-template <int L, bool MIXED>
-constexpr int warp_tpb() { return L == 16 && !MIXED ? 128 : 64; }
+// small requests launches half the CTAs (8,192 FP64 systems of n = 2..16 by
+// Newton 479 -> 446 us, by backtracking 485 -> 447; n = 2..12 382 -> 363).  Not
+// Rosenbrock's, whose pass counts spread widely (1,024 of n = 10: 1,323 us, 1,343
+// with four).
+template <int L, int FAM, bool MIXED>
+constexpr int warp_tpb() { return L == 16 && !MIXED && FAM != FAM_ROSENBROCK ? 128 : 64; }
 
 // One segment's shared memory.  U holds the pivot row of every step k, from
 // its column k on (the factor U by positions), at slot VEC - 1 + (column - k),
@@ -116,6 +118,7 @@ struct WarpSolver {
     using K = decltype(mag_bits(P(0)));
     using SM = WarpSmem<L, MIXED, FAM>;
     static constexpr int VEC = SM::VEC;
+    static constexpr int FAMILY = FAM;
 
     // ---- per-lane data of the current instance
     int r;         // row owned by this lane (0..L-1)
@@ -656,7 +659,7 @@ struct WarpSolver {
 template <int L, bool MIXED, int FAM>
 constexpr int warp_smem_bytes()
 {
-    constexpr int bytes = (warp_tpb<L, MIXED>() / 32) * (32 / L) * (int)sizeof(WarpSmem<L, MIXED, FAM>);
+    constexpr int bytes = (warp_tpb<L, FAM, MIXED>() / 32) * (32 / L) * (int)sizeof(WarpSmem<L, MIXED, FAM>);
     static_assert(bytes <= 48 * 1024, "no opt-in beyond 48 KB is made for these kernels");
     return bytes;
 }
@@ -685,7 +688,7 @@ NLS_DI void warp_lanes(SolveArgs &a)
     bool have = false, exhausted = false, first = true;
     int64_t k = -1;
     unsigned long long local_solved = 0;
-    const int64_t warp_global = (int64_t)blockIdx.x * (warp_tpb<L, MIXED>() / 32) + warp;
+    const int64_t warp_global = (int64_t)blockIdx.x * (warp_tpb<L, S::FAMILY, MIXED>() / 32) + warp;
 
     for (;;) {
         // segments are the units of work: one ballot bit per segment leader
@@ -760,12 +763,13 @@ template <int L, int FAM, bool MIXED>
 constexpr int warp_min_ctas()
 {
     if (L == 32) return MIXED ? 0 : 6;
-    if (L == 16) return !MIXED ? 4 : FAM == FAM_CUBIC ? 0 : 12;
+    if (L == 16 && MIXED) return FAM == FAM_CUBIC ? 0 : 12;
+    if (L == 16) return FAM == FAM_ROSENBROCK ? 0 : 4;
     return 0;
 }
 
 template <int L, int FAM, bool MIXED>
-__global__ void __launch_bounds__((warp_tpb<L, MIXED>()), (warp_min_ctas<L, FAM, MIXED>())) k_solve_warp(SolveArgs a)
+__global__ void __launch_bounds__((warp_tpb<L, FAM, MIXED>()), (warp_min_ctas<L, FAM, MIXED>())) k_solve_warp(SolveArgs a)
 {
     warp_lanes<WarpSolver<L, FAM, MIXED>, L, MIXED>(a);
 }

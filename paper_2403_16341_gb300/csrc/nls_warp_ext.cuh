@@ -374,7 +374,7 @@ constexpr int warp_ext_min_ctas()
 }
 
 template <int L, int FAM, bool MIXED, int ALG>
-__global__ void __launch_bounds__((warp_tpb<L, MIXED>()), (warp_ext_min_ctas<L, FAM, MIXED, ALG>())) k_solve_warp_ext(SolveArgs a)
+__global__ void __launch_bounds__((warp_tpb<L, FAM, MIXED>()), (warp_ext_min_ctas<L, FAM, MIXED, ALG>())) k_solve_warp_ext(SolveArgs a)
 {
     warp_lanes<typename warp_ext_solver<L, FAM, MIXED, ALG>::type, L, MIXED>(a);
 }
@@ -382,7 +382,7 @@ __global__ void __launch_bounds__((warp_tpb<L, MIXED>()), (warp_ext_min_ctas<L, 
 template <int L, int FAM, bool MIXED, int ALG>
 cudaError_t launch_warp_ext(const SolveArgs &a, int grid, cudaStream_t st)
 {
-    k_solve_warp_ext<L, FAM, MIXED, ALG><<<grid, warp_tpb<L, MIXED>(), warp_smem_bytes<L, MIXED, FAM>(), st>>>(a);
+    k_solve_warp_ext<L, FAM, MIXED, ALG><<<grid, (warp_tpb<L, FAM, MIXED>()), warp_smem_bytes<L, MIXED, FAM>(), st>>>(a);
     return cudaGetLastError();
 }
 
@@ -392,9 +392,9 @@ KernelInfo warp_ext_info()
     KernelInfo k;
     k.launch = &launch_warp_ext<L, FAM, MIXED, ALG>;
     k.func = reinterpret_cast<const void *>(&k_solve_warp_ext<L, FAM, MIXED, ALG>);
-    k.block = warp_tpb<L, MIXED>();
+    k.block = warp_tpb<L, FAM, MIXED>();
     k.smem = warp_smem_bytes<L, MIXED, FAM>();
-    k.per_cta = (warp_tpb<L, MIXED>() / 32) * (32 / L);
+    k.per_cta = (warp_tpb<L, FAM, MIXED>() / 32) * (32 / L);
     return k;
 }
 

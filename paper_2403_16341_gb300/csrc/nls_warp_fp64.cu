@@ -7,7 +7,7 @@ namespace nls {
 template <int L, int FAM>
 static cudaError_t launch_warp_fp64(const SolveArgs &a, int grid, cudaStream_t st)
 {
-    k_solve_warp<L, FAM, false><<<grid, warp_tpb<L, false>(), warp_smem_bytes<L, false, FAM>(), st>>>(a);
+    k_solve_warp<L, FAM, false><<<grid, (warp_tpb<L, FAM, false>()), warp_smem_bytes<L, false, FAM>(), st>>>(a);
     return cudaGetLastError();
 }
 
@@ -17,7 +17,7 @@ static KernelInfo info_fp64()
     KernelInfo k;
     k.launch = &launch_warp_fp64<L, FAM>;
     k.func = reinterpret_cast<const void *>(&k_solve_warp<L, FAM, false>);
-    k.block = warp_tpb<L, false>();
+    k.block = warp_tpb<L, FAM, false>();
     k.smem = warp_smem_bytes<L, false, FAM>();
     // An SM's split between L1 and shared memory changes only when the SM is idle,
     // and the driver takes the smallest split that a kernel's occupancy needs.
@@ -26,7 +26,7 @@ static KernelInfo info_fp64()
     // 664 systems, then cubic n = 32, 279: 627 us, 321 in the other order).  With
     // one split for all 32-lane kernels: 321 us in both.
     k.widest_smem = L == 32;
-    k.per_cta = (warp_tpb<L, false>() / 32) * (32 / L);
+    k.per_cta = (warp_tpb<L, FAM, false>() / 32) * (32 / L);
     return k;
 }
 

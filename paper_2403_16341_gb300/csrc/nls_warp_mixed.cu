@@ -7,7 +7,7 @@ namespace nls {
 template <int L, int FAM>
 static cudaError_t launch_warp_mixed(const SolveArgs &a, int grid, cudaStream_t st)
 {
-    k_solve_warp<L, FAM, true><<<grid, warp_tpb<L, true>(), warp_smem_bytes<L, true, FAM>(), st>>>(a);
+    k_solve_warp<L, FAM, true><<<grid, (warp_tpb<L, FAM, true>()), warp_smem_bytes<L, true, FAM>(), st>>>(a);
     return cudaGetLastError();
 }
 
@@ -17,9 +17,9 @@ static KernelInfo info_mixed()
     KernelInfo k;
     k.launch = &launch_warp_mixed<L, FAM>;
     k.func = reinterpret_cast<const void *>(&k_solve_warp<L, FAM, true>);
-    k.block = warp_tpb<L, true>();
+    k.block = warp_tpb<L, FAM, true>();
     k.smem = warp_smem_bytes<L, true, FAM>();
-    k.per_cta = (warp_tpb<L, true>() / 32) * (32 / L);
+    k.per_cta = (warp_tpb<L, FAM, true>() / 32) * (32 / L);
     return k;
 }
 
