@@ -40,7 +40,7 @@ constexpr int CTA_NMAX = 128;
 template <bool MIXED>
 struct CtaSmem {
     using P = typename std::conditional<MIXED, float, double>::type;
-    double u[CTA_NMAX], F[CTA_NMAX], dN[CTA_NMAX], ut[CTA_NMAX], Ft[CTA_NMAX];
+    double u[CTA_NMAX], F[CTA_NMAX], ut[CTA_NMAX];
     P Fp[CTA_NMAX], g[CTA_NMAX], Jg[CTA_NMAX], rhs[CTA_NMAX];
     P lcol[2][CTA_NMAX];    // multipliers of step k in buffer k & 1
     P rdiag[CTA_NMAX], x[CTA_NMAX];
