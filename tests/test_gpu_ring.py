@@ -115,3 +115,36 @@ def test_captured_flush_replays_beside_direct_ones(lone):
         replay()
         st.synchronize()
         solver.close()
+
+
+def test_entries_are_zero_again_on_the_second_lap(solver):
+    # two laps of the same layout: groups, lone requests of several waves (whose
+    # work counters end above their batch) and now and then a host request on
+    # both solve streams; a counter that is not zeroed again would have the
+    # grids of the second lap skip their instances
+    import paper_2403_16341_gb300 as nls
+    solver.set_option(nls.NLS_OPT_CTAS_PER_SM, 1)
+    small, waves, big = I.square_batch(2, 5), I.square_batch(2, 6000), I.square_batch(2, 1 << 18)
+    sp, su0 = on_gpu(small)
+    wp, wu0 = on_gpu(waves)
+    us = [su0.clone() for _ in range(500)]
+    wu = wu0.clone()
+    want, want_host = np.sqrt(waves.params), np.sqrt(big.params)
+    for lap in range(2):
+        for turn in range(64):
+            for v in us:
+                v.copy_(su0)
+            reqs = [solver.submit(nls.NLS_SQUARE, sp, v, NEWTON) for v in us[: 500 - 2 * (turn % 16 == 5)]]
+            solver.flush()
+            if turn % 16 == 5:
+                hu = big.u0.copy()
+                nls.nls_solve_host(solver.h, big.family, big.params.ctypes.data, hu.ctypes.data, big.n, big.batch, NEWTON,
+                                   1e-10, 50)
+                assert np.abs(hu - want_host).max() < 1e-9
+            for _ in range(12):
+                wu.copy_(wu0)
+                r = solver.submit(nls.NLS_SQUARE, wp, wu, NEWTON)
+                solver.flush()
+                assert solver.wait(r) == waves.batch, (lap, turn)
+            assert np.abs(wu.cpu().numpy() - want).max() < 1e-9
+            assert [solver.wait(r) for r in reqs] == [small.batch] * len(reqs), (lap, turn)
