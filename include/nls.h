@@ -204,7 +204,11 @@ int nls_solve(nls_handle h, int family, const double *params, double *u, int n, 
 int nls_adjoint(nls_handle h, int family, const double *params, const double *u, int n,
                 int64_t batch, const double *w, double *grad, int32_t *status);
 
-/* Launch every pending request of the handle on its stream (asynchronous). */
+/* Launch every pending request of the handle on its stream (asynchronous).
+ * While that stream is being captured, the launches and the zeroing of their
+ * counters are recorded instead: every replay solves from what u holds then.
+ * Launch each kernel once before the capture; nls_status cannot complete a
+ * captured request (its outputs are ready when the replay is). */
 int nls_flush(nls_handle h);
 
 /* Completion of request `req`: flushes if needed, then waits up to
