@@ -477,11 +477,12 @@ static int launch_graph(nls_batch *h, const std::vector<Request *> &rs, const st
 // 4,096 97.0 / 86.5).  A thread-tiled warp adds 32 instances at once and the
 // warps end apart: equal at 1,024 and 4,096 adds (cubic n = 3, 32,768: 55.0 / 54.8,
 // 131,072: 98.4 / 98.5), ahead where a refill spreads the ends (square n = 8).
+// CTA-tiled instances take long enough to end apart (Bratu, mixed, n = 64, 1,000:
+// 346 / 354, n = 96 823 / 834).
 static bool counts_in_mirror(const Request &r, int grid)
 {
-    if (r.tiles == NLS_TILE_THREAD) return grid <= 4096; // CTAs of one warp
     if (r.tiles == NLS_TILE_WARP) return (int64_t)grid * r.kern.block / 32 <= 512;
-    return r.args.batch <= 512;
+    return grid <= 4096;
 }
 
 static int launch_direct(nls_batch *h, const std::vector<Request *> &rs, const std::vector<int> &grids, int s0,
