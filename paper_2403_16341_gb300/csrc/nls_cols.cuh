@@ -44,7 +44,7 @@
 
 #include <climits>
 
-#include "nls_common.cuh"
+#include "nls_pivot.cuh"
 
 namespace nls {
 

@@ -53,7 +53,7 @@
 
 #include <climits>
 
-#include "nls_common.cuh"
+#include "nls_pivot.cuh"
 
 namespace nls {
 
