@@ -189,7 +189,7 @@ static int dev_alloc(nls_batch *h, void **p, size_t bytes)
 static KernelInfo cta_choice(const nls_batch *h, int family, int n, int alg, int64_t instances)
 {
     const bool mixed = (alg & NLS_MIXED) != 0;
-    if (mixed && instances <= nls::panel_most(family, n, (alg & NLS_REFINE) != 0, h->sms))
+    if (mixed && instances <= nls::panel_most(family, n, (alg & NLS_REFINE) != 0, false, h->sms))
         return nls::panel_kernel(family, n);
     return cta_kernel(family, n, mixed);
 }
@@ -359,21 +359,39 @@ static int default_refill(const nls_batch *h, int family, int alg)
 // grids leaves SMs idle when only a few kernels run concurrently).
 static int plan_grids(nls_batch *h, const std::vector<Request *> &rs, std::vector<int> &grids)
 {
+    // CTA-tiled mixed requests of the Newton family: panels or columns by the
+    // instances that they have together.  Side by side the two are slower than
+    // either, so the panels want every request within its line (600 Bratu systems of
+    // n = 40..80: 773 us mixed up, 654 on the columns); the cubic's, whose sizes wait
+    // for one another on the columns, only that none is too large for panels (300 of
+    // n = 90..120: 1.59 ms, 1.10 on the columns; but 2,048 of n = 33..48 908 us, 994).
     int live = 0;
-    int64_t cta_instances = 0; // mixed precision, Newton family
+    int64_t cta_instances = 0;
+    bool all_within = true, any_too_large = false;
     auto panel_or_columns = [](const Request &r) {
-        return r.tiles == NLS_TILE_CTA && (r.alg_flags & NLS_MIXED) && r.args.alg < NLS_POTRA_PTAK;
+        return r.tiles == NLS_TILE_CTA && (r.alg_flags & NLS_MIXED) && r.args.alg < NLS_POTRA_PTAK &&
+               r.args.batch > 0 && !r.poly;
+    };
+    for (Request *r : rs) {
+        if (r->args.batch > 0 && !r->poly) ++live;
+        if (panel_or_columns(*r)) cta_instances += r->args.batch;
+    }
+    auto within = [&](const Request &r) {
+        return cta_instances <= nls::panel_most(r.family, r.args.n, r.args.refine != 0, live > 1, h->sms);
     };
     for (Request *r : rs)
-        if (r->args.batch > 0 && !r->poly) {
-            ++live;
-            if (panel_or_columns(*r)) cta_instances += r->args.batch;
+        if (panel_or_columns(*r)) {
+            all_within = all_within && within(*r);
+            any_too_large = any_too_large || r->args.n > nls::PANEL_NMAX;
         }
     grids.assign(rs.size(), 0);
     for (size_t i = 0; i < rs.size(); ++i) {
         Request &r = *rs[i];
         if (r.args.batch == 0 || r.poly) continue; // a poly request runs its own chain
-        if (panel_or_columns(r)) r.kern = cta_choice(h, r.family, r.args.n, r.alg_flags, cta_instances);
+        if (panel_or_columns(r))
+            r.kern = within(r) && (r.family == FAM_CUBIC ? !any_too_large : all_within)
+                         ? nls::panel_kernel(r.family, r.args.n)
+                         : cta_kernel(r.family, r.args.n, true);
         int rc = prepare_kernel(h, r.kern);
         if (rc) return rc;
         const int64_t ctas = (r.args.batch + r.kern.per_cta - 1) / r.kern.per_cta;

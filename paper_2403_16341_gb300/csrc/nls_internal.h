@@ -60,16 +60,20 @@ KernelInfo panel_kernel(int family, int n);
 // end and beyond: Bratu n = 64 608: 0.80, 1,000: 1.20; n = 48 0.89, 1.30; n = 96 304:
 // 0.91, 456: 1.37; cubic n = 96 0.76, 1.23.  The cubic up to n = 64 re-reads A with
 // more threads per instance here, and stays ahead for more waves: n = 33 1,000: 0.91,
-// 2,000: 1.07; n = 48 2,000: 0.95, 4,000: 1.03; n = 64 2,000: 0.93, 4,000: 0.99;
+// 2,000: 1.07; n = 48 2,000: 0.95, 4,000: 1.03; n = 64 2,000: 0.93, 3,000: 0.94,
+// 4,000: 0.99;
 // refined n = 48 and 64 1,000: 0.90 and 0.86, 2,000: 1.05 and 1.00; n = 32 2,000: 0.93,
 // n = 24 608: 0.69, 1,000: 1.12.  The smallest systems (refined, or asked for) are one
 // panel there and gain nothing: 50 systems of n = 8 0.91 (cubic) and 1.03 (Bratu),
 // n = 16 0.73 and 0.86.
-inline int64_t panel_most(int family, int n, bool refine, int sms)
+// In a flush of several requests the cubic's larger sizes stay on the panels for
+// four waves (1,024 of n = 40..70 1.02 ms, 1.11 with n > 64 on the columns).
+constexpr int PANEL_NMAX = 96;
+inline int64_t panel_most(int family, int n, bool refine, bool several, int sms)
 {
     const bool cubic = family == FAM_CUBIC;
-    if (n > 96 || n < (cubic ? 8 : 9)) return 0;
-    const int waves = !cubic || n < 32 || n > 64 ? 1 : refine || n <= 40 ? 2 : 4;
+    if (n > PANEL_NMAX || n < (cubic ? 8 : 9)) return 0;
+    const int waves = !cubic || n < 32 ? 1 : n > 64 ? (several ? 4 : 1) : refine || n <= 40 ? 2 : 5;
     return (int64_t)waves * (n <= 64 ? 4 : 2) * sms;
 }
 } // namespace nls

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 NEWTON, LS, TR = 0, 1, 2
 MIXED, TILE_CTA, REFINE = 1 << 8, 1 << 12, 1 << 14
-MOST = 16  # waves of four or two CTAs per SM: no family stays on the panels above this many instances per SM
+MOST = 20  # instances per SM: above five waves of four CTAs no family stays on the panels
 
 
 @pytest.fixture(scope="module")

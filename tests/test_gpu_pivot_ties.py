@@ -78,7 +78,7 @@ def test_pivot_among_equals(solver, n, tiling, many, low_words, mixed):
         pytest.skip("one FP64 kernel serves all batches")
     B = 7
     A, b = paired(n, B, low_words)
-    reps = (2600 if n <= 64 else 700) // B if many else 1
+    reps = (3200 if n <= 64 else 700) // B if many else 1
     g = gpu_solve(solver, I.Batch(I.FAMILY_CUBIC, n, np.tile(np.concatenate([A.reshape(n * n, B), b]), (1, reps)),
                                   np.zeros((n, B * reps))), NEWTON | mixed | tiling, abstol=0.0, maxiters=1)
     ties = 0
